@@ -51,19 +51,28 @@ __device__ __forceinline__ void chord_normal(const float* pr, float& nxv, float&
     else { nxv = 1.f; nyv = 0.f; }
 }
 
-// Calls f(voxel, length) for every piece of segment P -> Q inside the grid.  The segment is
-// clipped to the grid, the crossings of the three plane families are merged in order of
-// their parameter t (each from its plane index: t = (o + k h - P) / D, computed with the
-// reciprocal of D), and a piece between consecutive crossings is credited to the voxel
-// between those planes: the voxel before the first crossing of each axis follows from
-// that crossing's plane index, and the index is stepped by one along the axis of every
-// crossing, so the voxel of a piece is always the one bounded by the planes around it
-// (the voxel holding the piece's midpoint).
-template <typename F>
-__device__ __forceinline__ void trace_segment(const Grid3& g, const float P[3], const float Q[3], F&& f) {
+// The pieces of one straight segment P -> Q inside the grid, in order.  The segment is clipped
+// to the grid, and each axis has its crossings as an arithmetic sequence of parameters: the
+// first from its plane index, t = (o + k h - P) / D, the j-th one j h / |D| later (a counter
+// and one FMA, so that nothing accumulates).  Only planes inside the grid are crossings (an
+// axis whose crossings are used up has t = 2), and their number is fixed before the walk, so
+// the number of pieces is known in advance and the voxel, stepped by one along the axis of
+// every crossing, stays inside the grid whatever the rounding of t.  The internal voxel index
+// is a sum of three terms: x keeps its term with the bits of the tile's y offset free, so that
+// a step is an add whose carry (or borrow) runs over those bits and a mask; y's term is formed
+// from its index; z's steps by a slice.
+struct Walk {
+    float t0, hi, L;
+    float t[3], a[3], d[3], j[3], c[3];   // next crossing, first, spacing, crossings done, their number
+    int fx, iy, fy, fz;   // x term, y index and its term, z term
+    int sx, sy, sz;       // steps of fx, iy and fz
+};
+
+// pieces of the segment (0: outside the grid); w is left at the first one
+__device__ __forceinline__ int walk_begin(const Grid3& g, const float P[3], const float Q[3], Walk& w) {
     const float D[3] = {Q[0] - P[0], Q[1] - P[1], Q[2] - P[2]};
-    const float L = sqrtf(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
-    if (!(L > 0.f)) return;
+    w.L = sqrtf(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
+    if (!(w.L > 0.f)) return 0;
     const float o[3] = {g.ox, g.oy, g.oz}, h[3] = {g.hx, g.hy, g.hz}, ih[3] = {g.ihx, g.ihy, g.ihz};
     const int n[3] = {g.nx, g.ny, g.nz};
     float inv[3];
@@ -73,55 +82,87 @@ __device__ __forceinline__ void trace_segment(const Grid3& g, const float P[3], 
         const float e0 = o[a], e1 = o[a] + n[a] * h[a];
         inv[a] = D[a] != 0.f ? 1.f / D[a] : 0.f;
         if (D[a] == 0.f) {
-            if (P[a] < e0 || P[a] > e1) return;
+            if (P[a] < e0 || P[a] > e1) return 0;
         } else {
-            float s0 = (e0 - P[a]) * inv[a], s1 = (e1 - P[a]) * inv[a];
-            if (s0 > s1) { const float t = s0; s0 = s1; s1 = t; }
-            lo = fmaxf(lo, s0);
-            hi = fminf(hi, s1);
+            const float s0 = (e0 - P[a]) * inv[a], s1 = (e1 - P[a]) * inv[a];
+            lo = fmaxf(lo, fminf(s0, s1));
+            hi = fminf(hi, fmaxf(s0, s1));
         }
     }
-    if (!(hi > lo)) return;
-    // next crossing of each axis: plane index k, parameter tn
-    int k[3], step[3];
-    float tn[3];
+    if (!(hi > lo)) return 0;
+    w.t0 = lo;
+    w.hi = hi;
+    int idx[3], total = 1;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (D[a] == 0.f) { tn[a] = 2.f; step[a] = 0; k[a] = 0; continue; }
-        const float u = (P[a] + lo * D[a] - o[a]) * ih[a];
-        step[a] = D[a] > 0.f ? 1 : -1;
-        k[a] = D[a] > 0.f ? (int)floorf(u) + 1 : (int)ceilf(u) - 1;
-        tn[a] = (o[a] + k[a] * h[a] - P[a]) * inv[a];
-        if (tn[a] <= lo) {   // the start lies on plane k: move to the next one
-            k[a] += step[a];
-            tn[a] = (o[a] + k[a] * h[a] - P[a]) * inv[a];
+        w.j[a] = 0.f;
+        w.d[a] = h[a] * fabsf(inv[a]);
+        w.a[a] = 2.f;
+        float c = 0.f;
+        if (D[a] == 0.f) {
+            idx[a] = min(max((int)floorf((P[a] - o[a]) * ih[a]), 0), n[a] - 1);
+        } else {
+            const float u = (P[a] + lo * D[a] - o[a]) * ih[a];
+            const bool up = D[a] > 0.f;
+            int k = up ? (int)floorf(u) + 1 : (int)ceilf(u) - 1;
+            if ((o[a] + k * h[a] - P[a]) * inv[a] <= lo) k += up ? 1 : -1;   // the start lies on plane k
+            k = up ? min(max(k, 1), n[a]) : min(max(k, 0), n[a] - 1);
+            w.a[a] = (o[a] + k * h[a] - P[a]) * inv[a];
+            // planes k .. n - 1 upwards, k .. 1 downwards; as many of them as lie before hi (one
+            // too many at most, which then makes an empty piece at hi)
+            if (w.a[a] < hi)
+                c = fminf((float)(up ? n[a] - k : k), ceilf((hi - w.a[a]) * fabsf(D[a]) * ih[a] + 1e-4f));
+            idx[a] = up ? k - 1 : k;
         }
+        w.c[a] = c;
+        w.t[a] = c > 0.f ? w.a[a] : 2.f;
+        total += (int)c;
     }
-    int idx[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int i = step[a] > 0 ? k[a] - 1 : step[a] < 0 ? k[a] : (int)floorf((P[a] - o[a]) * ih[a]);
-        idx[a] = min(max(i, 0), n[a] - 1);
+    w.iy = idx[1];
+    w.fx = grid_index(g, idx[0], 0, 0);
+    w.fy = grid_index(g, 0, idx[1], 0);
+    w.fz = idx[2] * g.slice_p;
+    w.sx = D[0] > 0.f ? 1 + (((1 << g.lty) - 1) << g.ltx) : -1;
+    w.sy = D[1] > 0.f ? 1 : -1;
+    w.sz = D[2] > 0.f ? g.slice_p : -g.slice_p;
+    return total;
+}
+
+// length of the current piece (0 when it is empty), then the step to the next one; v is the
+// piece's voxel
+__device__ __forceinline__ float walk_next(const Grid3& g, Walk& w, int& v) {
+    const float m = fminf(fminf(w.t[0], w.t[1]), w.t[2]), t1 = fminf(m, w.hi), dt = t1 - w.t0;
+    v = w.fx + w.fy + w.fz;
+    w.t0 = t1;
+    const bool px = w.t[0] == m, py = !px && w.t[1] == m;   // one axis steps; short enough to be predicated
+    if (px) {
+        w.fx = (w.fx + w.sx) & ~(((1 << g.lty) - 1) << g.ltx);
+        w.j[0] += 1.f;
+        w.t[0] = w.j[0] < w.c[0] ? fmaf(w.j[0], w.d[0], w.a[0]) : 2.f;
     }
-    float t0 = lo;
-    for (int guard = 0; guard < 4 * (g.nx + g.ny + g.nz) + 8; ++guard) {
-        int w = 0;
-        float t1 = tn[0];
-        if (tn[1] < t1) { t1 = tn[1]; w = 1; }
-        if (tn[2] < t1) { t1 = tn[2]; w = 2; }
-        const bool last = !(t1 < hi);
-        if (last) t1 = hi;
-        if (t1 - t0 > 1e-7f) f(grid_index(g, idx[0], idx[1], idx[2]), (t1 - t0) * L);
-        if (last) break;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {   // constant indices keep the arrays in registers
-            if (a == w) {
-                idx[a] = min(max(idx[a] + step[a], 0), n[a] - 1);
-                k[a] += step[a];
-                tn[a] = (o[a] + k[a] * h[a] - P[a]) * inv[a];
-            }
-        }
-        t0 = t1;
+    if (py) {
+        w.iy += w.sy;
+        w.fy = (w.iy << g.ltx) + (w.iy >> g.lty) * ((g.ntx - 1) << (g.ltx + g.lty));
+        w.j[1] += 1.f;
+        w.t[1] = w.j[1] < w.c[1] ? fmaf(w.j[1], w.d[1], w.a[1]) : 2.f;
+    }
+    if (!px && !py) {
+        w.fz += w.sz;
+        w.j[2] += 1.f;
+        w.t[2] = w.j[2] < w.c[2] ? fmaf(w.j[2], w.d[2], w.a[2]) : 2.f;
+    }
+    return dt > 1e-7f ? dt * w.L : 0.f;
+}
+
+// Calls f(voxel, length) for every piece of segment P -> Q inside the grid.
+template <typename F>
+__device__ __forceinline__ void trace_segment(const Grid3& g, const float P[3], const float Q[3], F&& f) {
+    Walk w;
+    const int n = walk_begin(g, P, Q, w);
+    for (int q = 0; q < n; ++q) {
+        int v;
+        const float l = walk_next(g, w, v);
+        if (l > 0.f) f(v, l);
     }
 }
 
@@ -208,93 +249,128 @@ __global__ void otf_rows_kernel(const float* __restrict__ paths, int64_t M, Grid
 }
 
 // ---------------------------------------------------------------- the DROP block
-// A group of 16 lanes per row (2 rows per warp); lane s traces segments s, s + 16, ...
-// The dot-product pass keeps the first kOtfCache accepted pieces of each lane (voxel,
-// length) in shared memory, and the scatter pass replays them; a lane with more pieces
-// traces its segments again and scatters only the pieces past the cached ones.
-// Four CTAs per SM: 64 registers per thread (no spills) and 4 x 48 KB of piece caches.
+// A warp takes two rows, 16 lanes each; lane s traces segments s, s + 16, ...  The pieces of
+// both rows are laid out along their paths in the warp's piece buffer in shared memory: a
+// segment's number of pieces is known before it is walked (walk_begin), so a prefix sum over
+// the lanes gives every lane its place.  The dot product and the scatter then read the buffer
+// with neighbouring lanes on neighbouring pieces, as the stored rows do: a gather or a
+// reduction of 16 consecutive pieces touches about 6 sectors of the tiled voxel order.  With
+// each lane on a segment of its own (the layout before this one) every lane touched a sector
+// of its own, and the L2's atomic sectors bounded the kernel: 262 us per 100k rows of the
+// 256x256x64 grid, 151 us with the buffer (issue slots 63 %, L2 42 %).
+// Pieces that are empty or shorter than min_len keep their place with length 0 and take no
+// part.  When a run of 16 segments a row does not fit into what is left of the buffer, it is
+// gathered and scattered piece by piece as it is traced (once for each).
 constexpr int kOtfThreads = 256;
-constexpr int kOtfCache = 24;
+constexpr int kOtfWarps = kOtfThreads / 32;
 
-__global__ void __launch_bounds__(kOtfThreads, 4) otf_drop_kernel(const float* __restrict__ paths,
-                                                                const float* __restrict__ b,
-                                                                const float* __restrict__ inv_norm2, int64_t r0,
-                                                                int64_t r1, Grid3 g, int n_seg, float min_len,
-                                                                const float* __restrict__ x, float* __restrict__ delta,
-                                                                float lambda, double* resid_ss) {
+// entries of a warp's buffer: two rows of a straight path across the grid with its segment
+// joins, in 72 KB (three CTAs per SM) or, when that suffices, 54 KB (four) a CTA
+static int otf_buffer(const OtfArgs& a) {
+    const int64_t need = 2 * ((int64_t)a.nx + a.ny + 2 * a.n_seg + 8);
+    return need <= 864 ? 864 : 1136;
+}
+
+template <int MINB>
+__global__ void __launch_bounds__(kOtfThreads, MINB) otf_drop_kernel(const float* __restrict__ paths,
+                                                                   const float* __restrict__ b,
+                                                                   const float* __restrict__ inv_norm2, int64_t r0,
+                                                                   int64_t r1, Grid3 g, int n_seg, float min_len,
+                                                                   const float* __restrict__ x,
+                                                                   float* __restrict__ delta, float lambda,
+                                                                   double* resid_ss, int cap) {
     constexpr int LPR = 16;
     extern __shared__ __align__(16) unsigned char otf_smem[];
-    int32_t* cv = reinterpret_cast<int32_t*>(otf_smem);                 // [kOtfCache][kOtfThreads]
-    float* cl = reinterpret_cast<float*>(cv + kOtfCache * kOtfThreads);  // [kOtfCache][kOtfThreads]
     const int tid = threadIdx.x;
-    const int lane = tid & 31, sub = lane % LPR;
+    const int lane = tid & 31, sub = lane % LPR, half = lane / LPR;
+    int2* buf = reinterpret_cast<int2*>(otf_smem) + (size_t)(tid >> 5) * cap;   // {voxel, length bits}
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + tid) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     double ss = 0.0;
     for (int64_t base = r0 + warp * 2; base < r1; base += nwarps * 2) {
-        const int64_t i = base + lane / LPR;
+        const int64_t i = base + half;
         const bool valid = i < r1;
-        float pr[10];
+        // the ends of segment sg of the row (the record is read again for every run of segments:
+        // kept in registers over the walk it spilled)
+        auto ends = [&](int sg, float A[3], float B[3]) {
+            float pr[10], nxv, nyv;
 #pragma unroll
-        for (int q = 0; q < 10; ++q) pr[q] = valid ? __ldg(paths + i * 10 + q) : 0.f;
-        float nxv, nyv;
-        chord_normal(pr, nxv, nyv);
+            for (int q = 0; q < 10; ++q) pr[q] = __ldg(paths + i * 10 + q);
+            chord_normal(pr, nxv, nyv);
+            path_point(pr, nxv, nyv, (float)sg / (float)n_seg, A);
+            path_point(pr, nxv, nyv, (float)(sg + 1) / (float)n_seg, B);
+        };
         float acc = 0.f;
-        int np = 0;   // accepted pieces of this lane
-        if (valid) {
-            for (int sg = sub; sg < n_seg; sg += LPR) {
+        int used = 0;   // the row's pieces in the buffer: the first row's from its start, the second's up to its end
+        int sg0 = 0;    // segments [0, sg0) are in the buffer
+        bool fits = true;
+        for (int s0 = 0; s0 < n_seg; s0 += LPR) {
+            const int sg = s0 + sub;
+            Walk w;
+            int n = 0;
+            if (valid && sg < n_seg) {
                 float A[3], B[3];
-                path_point(pr, nxv, nyv, (float)sg / (float)n_seg, A);
-                path_point(pr, nxv, nyv, (float)(sg + 1) / (float)n_seg, B);
-                trace_segment(g, A, B, [&](int v, float l) {
-                    if (l >= min_len) {
-                        if (np < kOtfCache) {
-                            cv[np * kOtfThreads + tid] = v;
-                            cl[np * kOtfThreads + tid] = l;
-                        } else {
-                            acc += l * __ldg(x + v);
-                        }
-                        ++np;
-                    }
-                });
+                ends(sg, A, B);
+                n = walk_begin(g, A, B, w);
             }
-            // the cached pieces' gathers are independent: issued back to back, four in flight
-            const int nc = np < kOtfCache ? np : kOtfCache;
-            int q = 0;
-            for (; q + 4 <= nc; q += 4) {
-                float xv[4], lv[4];
+            int at = n;   // inclusive prefix sum over the row's lanes
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    xv[u] = __ldg(x + cv[(q + u) * kOtfThreads + tid]);
-                    lv[u] = cl[(q + u) * kOtfThreads + tid];
+            for (int o = 1; o < LPR; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, at, o, LPR);
+                if (sub >= o) at += u;
+            }
+            const int tot = __shfl_sync(0xffffffffu, at, LPR - 1, LPR);
+            const int both = used + tot + __shfl_xor_sync(0xffffffffu, used + tot, LPR);
+            fits = fits && both <= cap;   // warp-uniform
+            if (fits) {
+                at = (half ? cap - used - tot : used) + at - n;
+                used += tot;
+                sg0 = s0 + LPR;
+                for (int q = 0; q < n; ++q) {
+                    int v;
+                    const float l = walk_next(g, w, v);
+                    buf[at + q] = make_int2(v, __float_as_int(l >= min_len ? l : 0.f));
                 }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) acc += lv[u] * xv[u];
+            } else {
+                for (int q = 0; q < n; ++q) {
+                    int v;
+                    const float l = walk_next(g, w, v);
+                    if (l > 0.f && l >= min_len) acc += l * __ldg(x + v);
+                }
             }
-            for (; q < nc; ++q) acc += cl[q * kOtfThreads + tid] * __ldg(x + cv[q * kOtfThreads + tid]);
+        }
+        __syncwarp();
+        const int2* mine = buf + (half ? cap - used : 0);
+        const int most = max(used, __shfl_xor_sync(0xffffffffu, used, LPR));
+        for (int q = sub; q < most; q += 4 * LPR) {   // four gathers in flight
+            float xv[4], lv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int2 e = q + u * LPR < used ? mine[q + u * LPR] : make_int2(0, 0);
+                lv[u] = __int_as_float(e.y);
+                xv[u] = lv[u] > 0.f ? __ldg(x + e.x) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc += lv[u] * xv[u];
         }
 #pragma unroll
         for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (!valid) continue;   // both halves of the warp are past their shuffles
-        const float res = __ldg(b + i) - acc;
-        const float r = lambda * res * __ldg(inv_norm2 + i);
-        if (sub == 0) ss += (double)res * (double)res;
-        const int nc = np < kOtfCache ? np : kOtfCache;
-        for (int q = 0; q < nc; ++q) atomicAdd(delta + cv[q * kOtfThreads + tid], r * cl[q * kOtfThreads + tid]);
-        if (np > kOtfCache) {
-            int seen = 0;
-            for (int sg = sub; sg < n_seg; sg += LPR) {
-                float A[3], B[3];
-                path_point(pr, nxv, nyv, (float)sg / (float)n_seg, A);
-                path_point(pr, nxv, nyv, (float)(sg + 1) / (float)n_seg, B);
-                trace_segment(g, A, B, [&](int v, float l) {
-                    if (l >= min_len) {
-                        if (seen >= kOtfCache) atomicAdd(delta + v, r * l);
-                        ++seen;
-                    }
-                });
-            }
+        const float res = valid ? __ldg(b + i) - acc : 0.f;
+        const float r = valid ? lambda * res * __ldg(inv_norm2 + i) : 0.f;
+        if (valid && sub == 0) ss += (double)res * (double)res;
+        for (int q = sub; q < used; q += LPR) {
+            const int2 e = mine[q];
+            const float l = __int_as_float(e.y);
+            if (l > 0.f) atomicAdd(delta + e.x, r * l);
         }
+        for (int sg = sg0 + sub; valid && sg < n_seg; sg += LPR) {   // segments past the buffer
+            float A[3], B[3];
+            ends(sg, A, B);
+            trace_segment(g, A, B, [&](int v, float l) {
+                if (l >= min_len) atomicAdd(delta + v, r * l);
+            });
+        }
+        __syncwarp();   // the buffer is read: the next rows may overwrite it
     }
     __shared__ double sh[32];
     const double tot = block_sum(ss, sh);
@@ -417,11 +493,14 @@ cudaError_t k_otf_prep(const OtfArgs& a, int64_t r0, int64_t r1, float* inv_norm
 cudaError_t k_otf_drop(const OtfArgs& a, int64_t r0, int64_t r1, const float* inv_norm2, const float* x, float* delta,
                        double lambda, double* resid_ss, cudaStream_t s) {
     if (r1 <= r0) return cudaSuccess;
-    const size_t smem = (size_t)kOtfCache * kOtfThreads * (sizeof(int32_t) + sizeof(float));
-    cudaError_t e = cudaFuncSetAttribute(otf_drop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int cap = otf_buffer(a);
+    const size_t smem = (size_t)cap * kOtfWarps * sizeof(int2);
+    auto kern = cap == 864 ? otf_drop_kernel<4> : otf_drop_kernel<3>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    otf_drop_kernel<<<a.grid, kOtfThreads, smem, s>>>(a.paths, a.b, inv_norm2, r0, r1, make_grid(a), a.n_seg,
-                                                      a.min_len, x, delta, (float)lambda, resid_ss);
+    const int grid = a.grid / 8 * (cap == 864 ? 4 : 3);   // a.grid: 8 CTAs per SM; one resident wave
+    kern<<<grid < 1 ? 1 : grid, kOtfThreads, smem, s>>>(a.paths, a.b, inv_norm2, r0, r1, make_grid(a), a.n_seg, a.min_len, x, delta,
+                                           (float)lambda, resid_ss, cap);
     return cudaGetLastError();
 }
 
