@@ -95,7 +95,8 @@ typedef struct {
  * with the matrix streamed into shared memory by the TMA engine (cp.async.bulk) ahead of
  * the consumer warps; needs 16-byte aligned col/val and 64 KB more shared memory.  When
  * the slice fits and rows come in runs of the same slice (e.g. stored by projection angle,
- * then slice), AUTO picks WINDOW (measured fastest); otherwise PLAIN.  Every schedule reads
+ * then slice), AUTO picks WINDOW (measured fastest); otherwise PLAIN.  With FP64
+ * arithmetic WINDOW keeps no window and scatters with global reductions (measured faster).  Every schedule reads
  * both index storages.  All give the same result up to the order of floating-point
  * summation. */
 #define NTVS_SCHED_AUTO 0

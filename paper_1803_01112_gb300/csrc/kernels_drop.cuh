@@ -123,13 +123,6 @@ struct WinScale {
     unsigned obs;
 };
 
-// Shared-memory slot of window offset j.  Paths along y step the offset by nx (200: 8
-// mod 32), which with slot = offset puts a warp's 32 updates into 4 banks; XORing the low
-// 5 bits with the next 5 (a bijection inside each group of 32 slots) spreads them.  The
-// FP32 path's internal voxel order already carries that swizzle inside each slice (the
-// window starts at a slice), so its slot is the offset itself; the FP64 path gathers the
-// canonical order and swizzles here.
-__device__ __forceinline__ int swz(int j) { return j ^ ((j >> 5) & 31); }
 // A DELTA16 word read without allocating in L1, which the x gathers then keep (0.2504 ->
 // 0.2481 ms per 500k-row BF16 block; the FP32 pairs measured slower this way, 0.2307 ->
 // 0.2325 ms, and keep the streaming load)
@@ -138,31 +131,19 @@ __device__ __forceinline__ uint32_t ld_no_l1(const uint32_t* p) {
     asm("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-template <typename T>
-__device__ __forceinline__ int win_slot(int j) {
-    if constexpr (sizeof(T) == 4) return j;
-    else return swz(j);
-}
-
-// delta_c += r * a.  In the window: FP32 compute adds round(rq * a) (rq = r / Q) to the
-// int32 fixed-point slot with a native shared-memory integer atomic when the row is
-// within the bound (rowfix), else the row's entries take the global path; FP64 compute
-// adds r * a to a double slot.  Outside the window: a global reduction.
+// delta_c += r * a.  In the window (FP32 compute): round(rq * a) (rq = r / Q) added to the int32
+// fixed-point slot, the offset itself (the internal voxel order carries the bank swizzle),
+// with a native shared-memory integer atomic when the row is within the bound (rowfix).
+// Everything else is a global reduction.
 template <typename T, bool WIN, bool D16>
 __device__ __forceinline__ void scatter(T* delta, const Window& w, int32_t c, T r, T a, bool rowfix, float rq) {
-    if (WIN) {
+    if constexpr (WIN) {
         const int rel = c - w.w0;
-        if ((unsigned)rel < (unsigned)w.W) {
-            if constexpr (sizeof(T) == 4) {
-                if (rowfix) {   // |rq a| < 2^22: adding 1.5 * 2^23 rounds it to the nearest integer
-                    const int y = __float_as_int(fmaf(rq, (float)a, 12582912.0f)) - 0x4B400000;
-                    atomicAdd(reinterpret_cast<int*>(window_base<T, D16>()) + win_slot<T>(rel), y);
-                    return;
-                }
-            } else {
-                atomicAdd(reinterpret_cast<T*>(window_base<T, D16>()) + win_slot<T>(rel), r * a);
-                return;
-            }
+        if ((unsigned)rel < (unsigned)w.W && rowfix) {
+            // |rq a| < 2^22: adding 1.5 * 2^23 rounds it to the nearest integer
+            const int y = __float_as_int(fmaf(rq, (float)a, 12582912.0f)) - 0x4B400000;
+            atomicAdd(reinterpret_cast<int*>(window_base<T, D16>()) + rel, y);
+            return;
         }
     }
     atomicAdd(delta + c, r * a);
@@ -177,7 +158,7 @@ __device__ __forceinline__ void row_factor(bool valid, bool first_lane, T res, T
     r = lambda * rn;
     rowfix = false;
     rq = 0.f;
-    if constexpr (WIN && sizeof(T) == 4) {
+    if constexpr (WIN) {
         const float arn = fabsf((float)rn);
         const float iq = ws->invQ;
         rowfix = iq > 0.f && arn <= ws->bound;
@@ -426,46 +407,31 @@ drop_block_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict
     if (threadIdx.x == 0 && tot != 0.0) atomicAdd(resid_ss, tot);
 }
 
-// Windowed variant: CTA b processes segments [seg_begin[b], seg_begin[b+1]) in order.
-// The window holds Wp = W rounded up to 32 slots (win_slot); slots past W stay 0.  FP32
-// compute keeps int32 multiples of the quantum Q, FP64 compute doubles.
+// Windowed variant (FP32 compute): CTA b processes segments [seg_begin[b], seg_begin[b+1]) in
+// order; the window holds int32 multiples of the quantum Q.
 // 4 consecutive floats added to global memory with one vector reduction (16-byte aligned)
 __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-template <typename T>
-__device__ __forceinline__ void flush_window(void* winp, int W, int Wp, T* delta, int w0, float Q) {
-    if constexpr (sizeof(T) == 4) {
-        int* win = reinterpret_cast<int*>(winp);
-        // slot j holds voxel w0 + j (win_slot<float> is the identity)
-        if (((w0 | W) & 3) == 0 && ((uintptr_t)delta & 15) == 0) {
-            // one 16-byte shared load and one vector reduction per four voxels
-            for (int j = 4 * threadIdx.x; j < W; j += 4 * blockDim.x) {
-                int4* slot = reinterpret_cast<int4*>(win + j);
-                const int4 v4 = *slot;
-                if ((v4.x | v4.y | v4.z | v4.w) == 0) continue;
-                red_add_v4(reinterpret_cast<float*>(delta) + w0 + j, (float)v4.x * Q, (float)v4.y * Q,
-                           (float)v4.z * Q, (float)v4.w * Q);
-                *slot = make_int4(0, 0, 0, 0);
-            }
-            return;
+__device__ __forceinline__ void flush_window(int* win, int W, float* delta, int w0, float Q) {
+    // slot j holds voxel w0 + j
+    if (((w0 | W) & 3) == 0 && ((uintptr_t)delta & 15) == 0) {
+        // one 16-byte shared load and one vector reduction per four voxels
+        for (int j = 4 * threadIdx.x; j < W; j += 4 * blockDim.x) {
+            int4* slot = reinterpret_cast<int4*>(win + j);
+            const int4 v4 = *slot;
+            if ((v4.x | v4.y | v4.z | v4.w) == 0) continue;
+            red_add_v4(delta + w0 + j, (float)v4.x * Q, (float)v4.y * Q, (float)v4.z * Q, (float)v4.w * Q);
+            *slot = make_int4(0, 0, 0, 0);
         }
-        for (int jj = threadIdx.x; jj < W; jj += blockDim.x) {
-            const int v = win[jj];
-            if (v != 0) {
-                atomicAdd(delta + w0 + jj, (float)v * Q);
-                win[jj] = 0;
-            }
-        }
-    } else {
-        T* win = reinterpret_cast<T*>(winp);
-        for (int jj = threadIdx.x; jj < Wp; jj += blockDim.x) {
-            const T v = win[jj];
-            if (v != (T)0) {
-                atomicAdd(delta + w0 + swz(jj), v);
-                win[jj] = (T)0;
-            }
+        return;
+    }
+    for (int jj = threadIdx.x; jj < W; jj += blockDim.x) {
+        const int v = win[jj];
+        if (v != 0) {
+            atomicAdd(delta + w0 + jj, (float)v * Q);
+            win[jj] = 0;
         }
     }
 }
@@ -478,16 +444,15 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
                          int64_t slice, const T* __restrict__ x, T* __restrict__ delta, T lambda,
                          double* resid_ss, Delta16 d16, const float* wlmax, const float* wbound, float* wobs,
                          const float* wamax) {
-    T* win = reinterpret_cast<T*>(window_base<T, D16>());
+    int* win = reinterpret_cast<int*>(window_base<T, D16>());
     const int W = (int)slice;
-    const int Wp = (W + 31) & ~31;
     __shared__ WinScale ws;
     __shared__ double ss_grp[32][32 / LPR];                     // per row group: sum of res^2 (one writer)
     constexpr int G = 32 / LPR;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
-    for (int j = threadIdx.x; j < Wp; j += blockDim.x) win[j] = (T)0;   // int 0 has the bits of 0.0f
+    for (int j = threadIdx.x; j < W; j += blockDim.x) win[j] = 0;
     for (int q = threadIdx.x; q < 32 * G; q += blockDim.x) (&ss_grp[0][0])[q] = 0.0;
     // rows with |r/lambda| <= bound keep |window slot| <= |lambda| bound lmax = 2^30 Q (no
     // int32 overflow); rows also below 2^22 Q / (|lambda| amax) keep every term below 2^22
@@ -496,7 +461,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
     const float Q = lam * bound * lmax * 0x1p-30f;
     if (threadIdx.x == 0) {
         const float iq = 1.f / Q;
-        const bool fix = sizeof(T) == 4 && bound > 0.f && amax > 0.f && Q > 0.f && isfinite(Q) && isfinite(iq);
+        const bool fix = bound > 0.f && amax > 0.f && Q > 0.f && isfinite(Q) && isfinite(iq);
         ws.invQ = fix ? iq : 0.f;
         ws.bound = fix ? fminf(bound, 0x1p22f * Q / (lam * amax)) : 0.f;
         ws.obs = 0u;
@@ -510,7 +475,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
         const DropSegment sg = segs[s];
         if (sg.home != cur) {   // uniform across the CTA
             __syncthreads();
-            flush_window<T>(win, W, Wp, delta, w.w0, Q);
+            flush_window(win, W, delta, w.w0, Q);
             __syncthreads();
             cur = sg.home;
             w.w0 = (int)(cur * slice);
@@ -564,7 +529,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
         }
     }
     __syncthreads();
-    flush_window<T>(win, W, Wp, delta, w.w0, Q);
+    flush_window(win, W, delta, w.w0, Q);
     if (lane < G) ss = ss_grp[warp][lane];
     __shared__ double sh[32];
     const double tot = block_sum(ss, sh);   // synchronizes the CTA
@@ -589,13 +554,12 @@ cudaError_t launch_window(const DropArgs& a, cudaStream_t s) {
 
 template <typename T, typename V, int LPR, int CH, int VW, bool D16>
 static cudaError_t launch_cfg(const DropArgs& a, cudaStream_t s) {
-    if (a.segs) {
-        return launch_window<T, V, LPR, CH, VW, D16>(a, s);
-    } else {
-        drop_block_kernel<T, V, LPR, CH, VW, D16><<<a.grid, 256, 0, s>>>(
-            a.row_ptr, a.col, (const V*)a.val, (const T*)a.b, (const T*)a.inv_norm2, a.r0, a.r1, (const T*)a.x,
-            (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16);
+    if constexpr (sizeof(T) == 4) {
+        if (a.segs) return launch_window<T, V, LPR, CH, VW, D16>(a, s);
     }
+    drop_block_kernel<T, V, LPR, CH, VW, D16><<<a.grid, 256, 0, s>>>(
+        a.row_ptr, a.col, (const V*)a.val, (const T*)a.b, (const T*)a.inv_norm2, a.r0, a.r1, (const T*)a.x,
+        (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16);
     return cudaGetLastError();
 }
 
