@@ -21,20 +21,38 @@
 
 namespace ntvs {
 
-template <typename T>
-__global__ void drop_apply_kernel(double* __restrict__ x, ImgCopies c, T* __restrict__ delta,
-                                  const T* __restrict__ inv_s, int64_t V, float* wbound, float* wobs) {
+template <typename T, int U>
+__global__ void __launch_bounds__(256) drop_apply_kernel(double* __restrict__ x, ImgCopies c, T* __restrict__ delta,
+                                                         const T* __restrict__ inv_s, int64_t V, float* wbound,
+                                                         float* wobs) {
     if (wbound && blockIdx.x == 0 && threadIdx.x == 0) {   // the window bound of the next sweep
         const float o = *wobs;
         if (o > 0.f) *wbound = 2.f * o;
         *wobs = 0.f;
     }
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < V; j += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = vox_internal(c.m, j);
-        const double v = x[j] + (double)delta[p] * (double)__ldg(inv_s + p);
-        x[j] = v;
-        store_copies(c, j, v);
-        delta[p] = (T)0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j0 < V; j0 += U * stride) {
+        double xv[U];
+        T dv[U], sv[U];
+        uint32_t p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = min(j0 + u * stride, V - 1);   // clamped: the loads issue together
+            p[u] = (uint32_t)vox_internal(c.m, j);
+            xv[u] = x[j];
+            dv[u] = delta[p[u]];
+            sv[u] = __ldg(inv_s + p[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = j0 + u * stride;
+            // an untouched voxel keeps its value and its gather copy
+            if (j >= V || (dv[u] == (T)0 && !c.xh)) continue;
+            const double v = xv[u] + (double)dv[u] * (double)sv[u];
+            x[j] = v;
+            store_copies(c, j, p[u], v);
+            delta[p[u]] = (T)0;
+        }
     }
 }
 
@@ -61,10 +79,13 @@ cudaError_t k_drop_block(const DropArgs& a, cudaStream_t s) {
 
 cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const void* inv_s, int64_t V, int grid,
                          float* wbound, float* wobs, cudaStream_t s) {
+    const bool many = vox_unrolled(V, grid);
     if (cdt == F64)
-        drop_apply_kernel<double><<<grid, 256, 0, s>>>(x, c, (double*)delta, (const double*)inv_s, V, wbound, wobs);
+        (many ? drop_apply_kernel<double, kVoxUnroll> : drop_apply_kernel<double, 1>)<<<grid, 256, 0, s>>>(
+            x, c, (double*)delta, (const double*)inv_s, V, wbound, wobs);
     else
-        drop_apply_kernel<float><<<grid, 256, 0, s>>>(x, c, (float*)delta, (const float*)inv_s, V, wbound, wobs);
+        (many ? drop_apply_kernel<float, kVoxUnroll> : drop_apply_kernel<float, 1>)<<<grid, 256, 0, s>>>(
+            x, c, (float*)delta, (const float*)inv_s, V, wbound, wobs);
     return cudaGetLastError();
 }
 

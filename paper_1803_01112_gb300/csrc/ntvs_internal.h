@@ -23,6 +23,22 @@ inline size_t dt_size(int dt) { return dt == F64 ? 8 : dt == F32 ? 4 : 2; }
 // offset in its slice.  tx = ty = 1 without sw is the canonical order (iz*ny + iy)*nx + ix.
 // Public images and the FP64 master stay canonical.  tx, ty are powers of two (ltx, lty
 // their logarithms); V and vint stay below 2^31.
+// u / d for u < 2^31 as a multiply and a shift: m = floor(2^(31+l) / d) + 1 with
+// l = ceil(log2 d) exceeds 2^(31+l) / d by less than 2^l / d, so u m / 2^(31+l) never reaches
+// the next integer; d = 1 keeps m = 0.
+struct FastDiv {
+    uint32_t m, s;
+};
+inline FastDiv make_fastdiv(uint32_t d) {
+    FastDiv f{0u, 0u};
+    if (d <= 1) return f;
+    uint32_t l = 1;
+    while (((uint64_t)1 << l) < d) ++l;
+    f.m = (uint32_t)((((uint64_t)1 << (31 + l)) / d) + 1);
+    f.s = l - 1;
+    return f;
+}
+
 struct VoxMap {
     int nx, ny, nz;
     int nxp, nyp;      // padded to multiples of tx, ty
@@ -31,6 +47,7 @@ struct VoxMap {
     int sw;            // 1: offsets swizzled inside each slice
     int64_t slice_p;   // nxp * nyp, rounded up to a multiple of 32 with sw
     int64_t vint;      // nz * slice_p
+    FastDiv dnx, dny;  // division by nx, ny
 };
 
 // tx, ty powers of two
@@ -48,6 +65,8 @@ inline VoxMap make_voxmap(int nx, int ny, int nz, int tx, int ty, bool sw = fals
     m.slice_p = (int64_t)m.nxp * m.nyp;
     if (sw) m.slice_p = (m.slice_p + 31) / 32 * 32;
     m.vint = m.slice_p * nz;
+    m.dnx = make_fastdiv((uint32_t)nx);
+    m.dny = make_fastdiv((uint32_t)ny);
     return m;
 }
 
