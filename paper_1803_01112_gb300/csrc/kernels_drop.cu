@@ -89,39 +89,78 @@ cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const voi
     return cudaGetLastError();
 }
 
-// out_i = <a_i, x> for rows [0, M), a warp per row (x in the gather order of the stored
-// columns), for CSR32 (packed pairs for FP32 values) or DELTA16 storage (words for 16-bit
-// values); accumulated in the compute type T.
+// out_i = <a_i, x> for rows [0, M) (x in the gather order of the stored columns), for CSR32
+// (packed pairs for FP32 values) or DELTA16 storage (words for 16-bit values); accumulated in
+// the compute type T, written as double when out64 is set, else as float.
+//
+// A warp takes 8 consecutive rows: their extents come with one load and their results leave
+// with one (row by row, a warp a row, each result was a 4-byte write to a sector of its own), and
+// while a row is summed the next one's lines are on their way to L2.  Up to 8 entries a lane
+// are loaded before their gathers, summed in the order of the entries.  2M rows of 255 FP32
+// pairs: 816 us with one row and one entry at a time, 684 us (0.94 of the measured copy rate).
+constexpr int kProjRows = 8, kProjStep = 8;
+
 template <typename T, typename V, bool D16>
 __global__ void __launch_bounds__(256)
 project_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, Delta16 d16,
-               const V* __restrict__ val, int64_t M, const T* __restrict__ x, T* __restrict__ out) {
+               const V* __restrict__ val, int64_t M, const T* __restrict__ x, void* __restrict__ out, int out64) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = w0; i < M; i += nw) {
-        const int64_t p0 = __ldg(row_ptr + i), p1 = __ldg(row_ptr + i + 1);
-        const int32_t* cbr = D16 ? d16.cbase + (p0 >> 5) + i : nullptr;
-        T acc = (T)0;
-        for (int64_t p = p0 + lane; p < p1; p += 32) {
-            int32_t c;
-            T a;
-            entry_any<T, V, D16>(col, d16, val, cbr, p, (int)(p - p0), c, a);
-            acc += a * __ldg(x + c);
+    for (int64_t base = w0 * kProjRows; base < M; base += nw * kProjRows) {
+        const int n = (int)min((int64_t)kProjRows, M - base);
+        const int64_t rp = lane <= n ? __ldg(row_ptr + base + lane) : 0;
+        T mine = (T)0;
+        for (int r = 0; r < n; ++r) {
+            const int64_t p0 = __shfl_sync(0xffffffffu, rp, r), p1 = __shfl_sync(0xffffffffu, rp, r + 1);
+            if constexpr (packed_entries<V, D16>()) {
+                const int64_t p2 = __shfl_sync(0xffffffffu, rp, min(r + 2, n));
+                prefetch_lines_l2(reinterpret_cast<const int2*>(col), p1, p2, lane);
+            }
+            const int32_t* cbr = D16 ? d16.cbase + (p0 >> 5) + base + r : nullptr;
+            T acc = (T)0;
+            for (int64_t p = p0 + lane; p < p1; p += 32 * kProjStep) {
+                int32_t c[kProjStep];
+                T a[kProjStep];
+#pragma unroll
+                for (int u = 0; u < kProjStep; ++u) {
+                    const int64_t q = p + 32 * u;
+                    c[u] = -1;
+                    a[u] = (T)0;
+                    if (q < p1) {
+                        if constexpr (packed_entries<V, D16>()) {
+                            const int2 e = __ldcs(reinterpret_cast<const int2*>(col) + q);
+                            c[u] = e.x;
+                            a[u] = (T)__int_as_float(e.y);
+                        } else {
+                            entry_any<T, V, D16>(col, d16, val, cbr, q, (int)(q - p0), c[u], a[u]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kProjStep; ++u)
+                    if (c[u] >= 0) acc += a[u] * __ldg(x + c[u]);
+            }
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == r) mine = acc;
         }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) out[i] = acc;
+        if (lane < n) {
+            if (out64) static_cast<double*>(out)[base + lane] = (double)mine;
+            else static_cast<float*>(out)[base + lane] = (float)mine;
+        }
     }
 }
 
 template <typename T, typename V>
-static cudaError_t launch_project(const DropArgs& a, int64_t M, const void* x, void* out, cudaStream_t s) {
+static cudaError_t launch_project(const DropArgs& a, int64_t M, const void* x, void* out, int out64, cudaStream_t s) {
+    const int64_t need = (M + 8 * kProjRows - 1) / (8 * kProjRows);   // 8 warps a CTA
+    const int grid = (int)(need < a.grid ? need : a.grid);
     if (a.use_d16)
-        project_kernel<T, V, true><<<a.grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M,
-                                                          (const T*)x, (T*)out);
+        project_kernel<T, V, true><<<grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M, (const T*)x, out,
+                                                        out64);
     else
-        project_kernel<T, V, false><<<a.grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M,
-                                                           (const T*)x, (T*)out);
+        project_kernel<T, V, false><<<grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M, (const T*)x,
+                                                         out, out64);
     return cudaGetLastError();
 }
 
@@ -155,17 +194,17 @@ cudaError_t k_pack_words(const uint16_t* off, const uint16_t* val, int64_t n, ui
     return cudaGetLastError();
 }
 
-cudaError_t k_project(const DropArgs& a, int64_t M, const void* x, void* out, cudaStream_t s) {
+cudaError_t k_project(const DropArgs& a, int64_t M, const void* x, void* out, int out64, cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
     if (a.cdt == F64) {
-        if (a.vdt == F64) return launch_project<double, double>(a, M, x, out, s);
-        if (a.vdt == F32) return launch_project<double, float>(a, M, x, out, s);
+        if (a.vdt == F64) return launch_project<double, double>(a, M, x, out, out64, s);
+        if (a.vdt == F32) return launch_project<double, float>(a, M, x, out, out64, s);
         return cudaErrorInvalidValue;
     }
     switch (a.vdt) {
-        case F32: return launch_project<float, float>(a, M, x, out, s);
-        case F16: return launch_project<float, __half>(a, M, x, out, s);
-        case BF16: return launch_project<float, __nv_bfloat16>(a, M, x, out, s);
+        case F32: return launch_project<float, float>(a, M, x, out, out64, s);
+        case F16: return launch_project<float, __half>(a, M, x, out, out64, s);
+        case BF16: return launch_project<float, __nv_bfloat16>(a, M, x, out, out64, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kOtfThreads, MINB) otf_drop_kernel(const float
 // i's path, the rows the DROP sweeps use; 16 lanes per row, each tracing every 16th segment.
 __global__ void __launch_bounds__(256) otf_project_kernel(const float* __restrict__ paths, int64_t M, Grid3 g,
                                                            int n_seg, float min_len, const float* __restrict__ x,
-                                                           float* __restrict__ out) {
+                                                           void* __restrict__ out, int out64) {
     constexpr int LPR = 16;
     const int lane = threadIdx.x & 31, sub = lane % LPR;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -426,7 +426,10 @@ __global__ void __launch_bounds__(256) otf_project_kernel(const float* __restric
         }
 #pragma unroll
         for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (valid && sub == 0) out[i] = acc;
+        if (valid && sub == 0) {
+            if (out64) static_cast<double*>(out)[i] = (double)acc;
+            else static_cast<float*>(out)[i] = acc;
+        }
     }
 }
 
@@ -536,9 +539,9 @@ cudaError_t k_otf_fill_rows(const OtfArgs& a, const int64_t* row_ptr, int32_t* c
     return cudaGetLastError();
 }
 
-cudaError_t k_otf_project(const OtfArgs& a, const float* x, float* out, cudaStream_t s) {
+cudaError_t k_otf_project(const OtfArgs& a, const float* x, void* out, int out64, cudaStream_t s) {
     if (a.M <= 0) return cudaSuccess;
-    otf_project_kernel<<<a.grid, 256, 0, s>>>(a.paths, a.M, make_grid(a), a.n_seg, a.min_len, x, out);
+    otf_project_kernel<<<a.grid, 256, 0, s>>>(a.paths, a.M, make_grid(a), a.n_seg, a.min_len, x, out, out64);
     return cudaGetLastError();
 }
 

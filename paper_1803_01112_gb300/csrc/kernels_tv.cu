@@ -282,6 +282,13 @@ __global__ void __launch_bounds__(kRedThreads) x32_from_x64_kernel(const double*
     }
 }
 
+// the gather image of canonical image src: out[internal(j)] = (float)src[j]
+template <typename S>
+__global__ void gather_image_kernel(const S* __restrict__ src, float* __restrict__ out, VoxMap m, int64_t V) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < V; j += (int64_t)gridDim.x * blockDim.x)
+        out[vox_internal(m, j)] = (float)src[j];
+}
+
 static int g_sm_count = 0;
 static int sm_count() {
     if (!g_sm_count) {
@@ -358,6 +365,14 @@ cudaError_t k_x32_from_x64(const double* x, ImgCopies c, cudaStream_t s) {
     const int64_t V = (int64_t)c.m.nx * c.m.ny * c.m.nz;
     const int grid = red_grid(V, sm_count());
     (vox_unrolled(V, grid) ? x32_from_x64_kernel<kVoxUnroll> : x32_from_x64_kernel<1>)<<<grid, kRedThreads, 0, s>>>(x, c);
+    return cudaGetLastError();
+}
+
+cudaError_t k_gather_image(const void* src, int sdt, float* out, const VoxMap& m, cudaStream_t s) {
+    const int64_t V = (int64_t)m.nx * m.ny * m.nz;
+    const int grid = red_grid(V, sm_count());
+    if (sdt == F64) gather_image_kernel<double><<<grid, 256, 0, s>>>((const double*)src, out, m, V);
+    else gather_image_kernel<float><<<grid, 256, 0, s>>>((const float*)src, out, m, V);
     return cudaGetLastError();
 }
 

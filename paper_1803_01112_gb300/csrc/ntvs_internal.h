@@ -119,6 +119,8 @@ cudaError_t k_colmax(const float* v, int64_t n, float* out, cudaStream_t s);
 cudaError_t k_remap_cols(const int32_t* col_in, int32_t* col_out, int64_t nnz, VoxMap m, int* flags, cudaStream_t s);
 // x32[internal(j)] = (float)x[j] for the canonical voxels j < V
 cudaError_t k_x32_from_x64(const double* x, ImgCopies c, cudaStream_t s);
+// out[internal(j)] = (float)src[j] (src: canonical, F64 or F32); padding slots are left alone
+cudaError_t k_gather_image(const void* src, int sdt, float* out, const VoxMap& m, cudaStream_t s);
 // inv_s[j] = cnt[j] ? 1/cnt[j] : 0
 cudaError_t k_inv_counts(const int32_t* cnt, void* inv_s, int cdt, int64_t n, cudaStream_t s);
 
@@ -251,8 +253,8 @@ cudaError_t k_chunk_cost(const int64_t* row_ptr, const int64_t* cs, const int8_t
                          int64_t* cost, int grid, cudaStream_t s);
 cudaError_t k_drop_block_d16(const DropArgs& a, cudaStream_t s);   // the same on DELTA16 storage
 // out[i] = <a_i, x> for the M rows (x: compute type, in the order of the stored columns;
-// out: compute type); a.row_ptr, col / d16, val, vdt, cdt, use_d16 and grid are used
-cudaError_t k_project(const DropArgs& a, int64_t M, const void* x, void* out, cudaStream_t s);
+// out: double when out64, else float); a.row_ptr, col / d16, val, vdt, cdt, use_d16 and grid are used
+cudaError_t k_project(const DropArgs& a, int64_t M, const void* x, void* out, int out64, cudaStream_t s);
 // *out = max(*out, longest row of rows [r0, r1)); *out zeroed by the caller
 cudaError_t k_row_maxlen(const int64_t* row_ptr, int64_t r0, int64_t r1, unsigned long long* out, int grid,
                          cudaStream_t s);
@@ -334,7 +336,7 @@ cudaError_t k_otf_prep(const OtfArgs& a, int64_t r0, int64_t r1, float* inv_norm
 cudaError_t k_otf_drop(const OtfArgs& a, int64_t r0, int64_t r1, const float* inv_norm2, const float* x, float* delta,
                        double lambda, double* resid_ss, cudaStream_t s);
 // out[i] = <a_i, x> of every traced row (x in the internal voxel order)
-cudaError_t k_otf_project(const OtfArgs& a, const float* x, float* out, cudaStream_t s);
+cudaError_t k_otf_project(const OtfArgs& a, const float* x, void* out, int out64, cudaStream_t s);
 // stored rows from paths: entries per row, then (voxel in the order of a.vm, length) from row_ptr
 cudaError_t k_otf_count_rows(const OtfArgs& a, int32_t* nnz_row, cudaStream_t s);
 cudaError_t k_otf_fill_rows(const OtfArgs& a, const int64_t* row_ptr, int32_t* col, float* val, cudaStream_t s);
