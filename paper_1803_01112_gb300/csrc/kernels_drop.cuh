@@ -503,20 +503,21 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
             for (int base = warp * G; base < n; base += nwarps * G) {
                 const int k = base + grp;
                 const bool valid = k < n;
-                if constexpr (kPrefetchRows > 0 && LPR == 32) {
-                    const int kp = k + kPrefetchRows * nwarps;   // this warp's row that many iterations ahead
+                if constexpr (kPrefetchRows > 0 && LPR >= 16) {
+                    const int kp = k + kPrefetchRows * nwarps * G;   // this group's row that many iterations ahead
+                    const int sub = lane % LPR;
                     if (kp < n) {
                         const int64_t q0 = stage_rp<T, D16>()[kp], q1 = stage_rp<T, D16>()[kp + 1];
                         if constexpr (D16) {
-                            if constexpr (delta16_words<V, D16>()) prefetch_lines_l2(d16.word, q0, q1, lane);
-                            else prefetch_row_l2(d16.off, val, q0, q1, lane);
+                            if constexpr (delta16_words<V, D16>()) prefetch_lines_l2(d16.word, q0, q1, sub);
+                            else prefetch_row_l2(d16.off, val, q0, q1, sub);
                             // and the chunk bases of a row that is not narrow (one short run)
-                            if (lane == 31 && !(stage_fl<T, D16>()[kp] & 2))
+                            if (sub == LPR - 1 && !(stage_fl<T, D16>()[kp] & 2))
                                 asm volatile("prefetch.global.L2 [%0];" ::"l"(d16.cbase + (q0 >> 5) + c0 + kp));
                         } else if constexpr (packed_entries<V, D16>()) {
-                            prefetch_lines_l2(reinterpret_cast<const int2*>(col), q0, q1, lane);
+                            prefetch_lines_l2(reinterpret_cast<const int2*>(col), q0, q1, sub);
                         } else {
-                            prefetch_row_l2(col, val, q0, q1, lane);
+                            prefetch_row_l2(col, val, q0, q1, sub);
                         }
                     }
                 }
@@ -570,6 +571,15 @@ static cudaError_t dispatch(const DropArgs& a, cudaStream_t s) {
     // longest row needs (window_register_steps: 8..12; longer rows finish in the tail loop),
     // so blocks of short rows do not evaluate empty steps; the schedule planner balances the
     // CTAs by the same rule
+    if constexpr (packed_entries<V, D16>() && sizeof(T) == 4) {
+        // Two rows a warp: a row's time is its chain of round trips, so rows that leave half of
+        // the 8-step body of 32 lanes empty go two at a time.  us per block with 32 lanes and
+        // with 16, rows of 132 entries (96x96x12): 21.9 / 21.0 at 25000 rows, 32.3 / 29.6 at
+        // 60000, 49.5 / 42.5 at 120000; rows of 175 (128x128x16): 23.6 / 25.0, 34.9 / 36.2 and
+        // 53.0 / 52.9, so the load takes 16 lanes up to a mean of 150.
+        if (a.segs && a.lanes_per_row == 16)
+            return a.max_row <= 160 ? launch_cfg<T, V, 16, 10, 1, D16>(a, s) : launch_cfg<T, V, 16, 12, 1, D16>(a, s);
+    }
     if constexpr (sizeof(T) == 4 && (std::is_same<V, float>::value || std::is_same<V, __nv_bfloat16>::value)) {
         if (a.segs) {
             switch (window_register_steps(a.max_row, a.cdt, a.vdt, a.lanes_per_row)) {

@@ -104,6 +104,7 @@ struct ntvs_ctx {
     void* inv_norm2 = nullptr;
     void* inv_s = nullptr;
     int lpr = 32;
+    int win_lpr = 32;                  // lanes per row of the windowed schedule
     int drop_grid = 1;
     int apply_grid = 1;
     bool vector4 = false;
@@ -553,7 +554,7 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
     a.resid_ss = resid;
     a.vdt = c->vdt;
     a.cdt = c->cdt;
-    a.lanes_per_row = c->lpr;
+    a.lanes_per_row = whole && c->schedule == NTVS_SCHED_WINDOW && c->segs ? c->win_lpr : c->lpr;
     a.grid = c->drop_grid;
     a.vector4 = c->vector4;
     a.use_d16 = c->storage == NTVS_DELTA16;
@@ -758,7 +759,7 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
     std::vector<int8_t> chunk_ch((size_t)std::max<int64_t>(nch, 1), 0);
     for (int t = 0; t < c->B; ++t) {
         const int64_t mr = t < (int)c->block_maxrow.size() ? c->block_maxrow[t] : 0;
-        const int8_t d = (int8_t)window_register_steps(mr, c->cdt, c->vdt, c->lpr);
+        const int8_t d = (int8_t)window_register_steps(mr, c->cdt, c->vdt, c->win_lpr);
         for (int64_t q = block_chunk[t]; q < block_chunk[t + 1]; ++q) chunk_ch[(size_t)q] = d;
     }
     // the planning's device temporaries in one allocation (each free synchronizes the device)
@@ -1348,6 +1349,8 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     // launch shapes: lanes per row from the mean row length
     const double mean = M ? (double)nnz / (double)M : 0.0;
     c->lpr = mean <= 12.0 ? 4 : mean <= 40.0 ? 8 : mean <= 120.0 ? 16 : 32;
+    // windowed FP32 pairs: two rows a warp up to a mean of 150 entries (kernels_drop.cuh, dispatch)
+    c->win_lpr = c->lpr == 32 && mean <= 150.0 && c->ent ? 16 : c->lpr;
     c->drop_grid = c->sms * 8;
     // 4-entry vector loads put entries 4 apart along a path into one scatter instruction,
     // which measured slower than one coalesced entry per lane (2-entry loads too: 0.312
