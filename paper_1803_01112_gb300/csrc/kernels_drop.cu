@@ -164,21 +164,6 @@ static cudaError_t launch_project(const DropArgs& a, int64_t M, const void* x, v
     return cudaGetLastError();
 }
 
-// ent[p] = {col[p], bits of val[p]} for entries [0, n)
-__global__ void pack_entries_kernel(const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n,
-                                    int2* __restrict__ ent) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-        ent[p] = make_int2(__ldcs(col + p), __float_as_int(__ldcs(val + p)));
-}
-
-cudaError_t k_pack_entries(const int32_t* col, const float* val, int64_t n, int32_t* ent, cudaStream_t s) {
-    if (n <= 0) return cudaSuccess;
-    const int64_t need = (n + 255) / 256;
-    const int grid = (int)(need < 4096 ? need : 4096);
-    pack_entries_kernel<<<grid, 256, 0, s>>>(col, val, n, reinterpret_cast<int2*>(ent));
-    return cudaGetLastError();
-}
-
 // word[p] = off[p] | val[p] << 16 (16-bit value bits) for entries [0, n)
 __global__ void pack_words_kernel(const uint16_t* __restrict__ off, const uint16_t* __restrict__ val, int64_t n,
                                   uint32_t* __restrict__ word) {

@@ -610,12 +610,12 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
 // One block-DROP step: this context's rows of block t into delta, the sum over ranks
 // through the all-reduce callback when one is set (row-sharded reconstruction), then
 // x += delta / s^t.
-int drop_block(ntvs_ctx* c, int t) {
+int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
     const int64_t r0 = c->block_ptr[t], r1 = c->block_ptr[t + 1];
     // the split copies of x are written by the last block of a sweep only (the TV gradient
     // reads them next); after any other block they are marked stale
     const bool split = t == c->B - 1;
-    CUDA_TRY(cudaMemsetAsync(c->resid + t, 0, sizeof(double), c->stream));
+    if (!resid_cleared) CUDA_TRY(cudaMemsetAsync(c->resid + t, 0, sizeof(double), c->stream));
     if (r1 <= r0 && !c->ar_fn) return NTVS_OK;
     float* wb = nullptr;
     float* wo = nullptr;
@@ -637,7 +637,8 @@ int drop_block(ntvs_ctx* c, int t) {
 }
 
 int drop_sweep(ntvs_ctx* c) {
-    for (int t = 0; t < c->B; ++t) TRY(drop_block(c, t));
+    CUDA_TRY(cudaMemsetAsync(c->resid, 0, sizeof(double) * (size_t)c->B, c->stream));
+    for (int t = 0; t < c->B; ++t) TRY(drop_block(c, t, true));
     return NTVS_OK;
 }
 
@@ -1224,7 +1225,10 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     // validation; columns of the internal order are rewritten into a buffer of the context's
     // own (caller memory is never modified)
     CUDA_TRY(cudaMemsetAsync(c->dflags, 0, sizeof(int), st));
-    if (reordered && nnz > 0 && !piped) {
+    // CSR32 storage with FP32 values: the preparation packs every block's entries into {column,
+    // value} pairs of the internal order itself (during the copy of the later blocks)
+    const bool pack = c->storage == NTVS_CSR32 && c->vdt == F32;
+    if (reordered && nnz > 0 && !piped && !pack) {
         if (!c->own_col) {
             int32_t* mine = nullptr;
             TRY(dev_alloc(&mine, sizeof(int32_t) * (size_t)nnz, "col (internal order)"));
@@ -1244,25 +1248,28 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     }
     // one pass per block: entry / rhs validation, FP64 row norms, per-block hit counts
     TRY(dev_alloc(&c->inv_norm2, csz * (size_t)M, "inv_norm2"));
+    // hit counts: integers for all blocks at once (FP64), or (FP32) one block's counts beside its
+    // column sums of |a_ij|, from which come the inverse counts and the scale statistics of the
+    // fixed-point DROP window (lmax = the largest column sum, the bound seeded with
+    // max_i |b_i| / ||a_i||^2)
     int32_t* cnt = nullptr;
-    TRY(dev_alloc(&cnt, sizeof(int32_t) * (size_t)c->B * VI, "hit counts"));
-    CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)c->B * VI, st));
-    // FP32 path: per-block scale statistics of the fixed-point DROP window (lmax = the
-    // largest column sum of |a_ij|, the bound seeded with max_i |b_i| / ||a_i||^2)
-    float* colsum = nullptr;
-    struct FreeColsum {
-        float*& p;
-        ~FreeColsum() { dev_free(p); }
-    } colsum_guard{colsum};
+    float2* cs = nullptr;
+    struct FreeCounts {
+        int32_t*& p;
+        float2*& q;
+        ~FreeCounts() { dev_free(p); dev_free(q); }
+    } counts_guard{cnt, cs};
+    TRY(dev_alloc(&c->inv_s, csz * (size_t)c->B * VI, "inverse hit counts"));
     if (c->cdt == F32) {
         TRY(dev_alloc(&c->wstat, sizeof(float) * 5 * (size_t)c->B, "window scale statistics"));
         CUDA_TRY(cudaMemsetAsync(c->wstat, 0, sizeof(float) * 5 * (size_t)c->B, st));
-        TRY(dev_alloc(&colsum, sizeof(float) * (size_t)VI, "column sums"));
+        TRY(dev_alloc(&cs, sizeof(float2) * (size_t)VI, "hit counts and column sums"));
+        CUDA_TRY(cudaMemsetAsync(cs, 0, sizeof(float2) * (size_t)VI, st));
+    } else {
+        TRY(dev_alloc(&cnt, sizeof(int32_t) * (size_t)c->B * VI, "hit counts"));
+        CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)c->B * VI, st));
     }
-    // CSR32 storage with FP32 values: every block's entries are packed into {column, value}
-    // pairs once they are validated and remapped (during the copy of the later blocks)
-    if (c->storage == NTVS_CSR32 && c->vdt == F32)
-        TRY(dev_alloc(&c->ent, sizeof(int32_t) * 2 * (size_t)std::max<int64_t>(nnz, 1), "packed entries"));
+    if (pack) TRY(dev_alloc(&c->ent, sizeof(int32_t) * 2 * (size_t)std::max<int64_t>(nnz, 1), "packed entries"));
     if (ring && !c->ent) return fail(NTVS_ERR_STATE, "staged load without packed entries");
     for (int t = 0; t < c->B; ++t) {
         // block t's entries: from entry e0 on at bc / bv (the whole arrays when not piped)
@@ -1275,15 +1282,12 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
             bc = block_col(t);
             bv = block_val(t);
             e0 = eb[t];
-            if (reordered) CUDA_TRY(k_remap_cols(bc, bc, eb[t + 1] - eb[t], c->vm, c->dflags, st));
+            if (reordered && !pack) CUDA_TRY(k_remap_cols(bc, bc, eb[t + 1] - eb[t], c->vm, c->dflags, st));
         }
-        if (colsum) CUDA_TRY(cudaMemsetAsync(colsum, 0, sizeof(float) * (size_t)VI, st));
-        CUDA_TRY(k_prep_block(c->row_ptr, bc, bv, e0, c->vdt, c->b, bp[t], bp[t + 1], VI, c->inv_norm2, c->cdt,
-                              cnt + (size_t)t * VI, c->dflags, colsum, colsum ? c->wstat + 3 * c->B + 2 * t : nullptr,
-                              st));
-        if (colsum) CUDA_TRY(k_colmax(colsum, VI, c->wstat + t, st));
-        if (c->ent && piped)
-            CUDA_TRY(k_pack_entries(bc, (const float*)bv, eb[t + 1] - eb[t], c->ent + 2 * eb[t], st));
+        CUDA_TRY(k_prep_block(c->row_ptr, bc, bv, e0, c->vdt, c->b, bp[t], bp[t + 1], pack ? V : VI, c->vm,
+                              c->inv_norm2, c->cdt, cnt ? cnt + (size_t)t * VI : nullptr, c->dflags, cs,
+                              cs ? c->wstat + 3 * c->B + 2 * t : nullptr, c->ent, st));
+        if (cs) CUDA_TRY(k_finish_block(cs, VI, (float*)c->inv_s + (size_t)t * VI, c->wstat + t, c->dflags, st));
         if (ring) {   // the slot is free again: the block nslots on may be copied into it
             cudaEvent_t ev;
             CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -1292,7 +1296,6 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
             if (t + nslots < c->B) TRY(issue_copy(t + nslots));
         }
     }
-    if (c->ent && !piped) CUDA_TRY(k_pack_entries(c->col, (const float*)c->val, nnz, c->ent, st));
     {   // longest row of every block
         unsigned long long* dm = nullptr;
         TRY(dev_alloc(&dm, sizeof(unsigned long long) * (size_t)c->B, "row lengths"));
@@ -1316,17 +1319,24 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     }
     CUDA_TRY(cudaMemcpyAsync(c->hint, c->dflags, sizeof(int), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
-    if (c->hint[0]) {
+    if (c->hint[0] & ~64) {
         const int f = c->hint[0];
-        dev_free(cnt);
         c->free_system();
         return fail(NTVS_ERR_CSR, (f & 4) ? "column index outside [0, V)" : (f & 8) ? "non-finite matrix value"
                                                                                     : "non-finite right-hand side");
     }
-    TRY(dev_alloc(&c->inv_s, csz * (size_t)c->B * VI, "inverse hit counts"));
-    CUDA_TRY(k_inv_counts(cnt, c->inv_s, c->cdt, (int64_t)c->B * VI, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    dev_free(cnt);
+    if (c->hint[0] & 64) {   // a voxel with 2^24 hits in a block or more: every block counted in integers
+        TRY(dev_alloc(&cnt, sizeof(int32_t) * (size_t)c->B * VI, "hit counts"));
+        CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)c->B * VI, st));
+        for (int t = 0; t < c->B; ++t) {
+            if (c->ent) CUDA_TRY(k_recount(c->row_ptr, bp[t], bp[t + 1], c->ent, cnt + (size_t)t * VI, st));
+            else
+                CUDA_TRY(k_prep_block(c->row_ptr, c->col, c->val, 0, c->vdt, c->b, bp[t], bp[t + 1], VI, c->vm,
+                                      c->inv_norm2, c->cdt, cnt + (size_t)t * VI, c->dflags, nullptr, nullptr, nullptr,
+                                      st));
+        }
+    }
+    if (cnt) CUDA_TRY(k_inv_counts(cnt, c->inv_s, c->cdt, (int64_t)c->B * VI, st));
 
     // image state (x and g canonical; x32 and delta in the internal order, padding zero)
     TRY(dev_alloc(&c->x, sizeof(double) * (size_t)V, "x"));

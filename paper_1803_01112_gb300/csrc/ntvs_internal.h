@@ -104,16 +104,21 @@ int red_grid(int64_t n, int sm_count);
 // ------------------------------------------------------------------ load-time prep
 // flags |= 1 if row_ptr decreases, 2 if row_ptr[0] != 0
 cudaError_t k_validate_rows(const int64_t* row_ptr, int64_t M, int* flags, cudaStream_t s);
-// fused pass over the rows [r0, r1) of one block: validation of columns, values and b
-// (flags 4 / 8 / 16), inv_norm2 of the rows and the block's hit counts cnt; with colsum
-// (nullable) also colsum[j] += |a_ij|, rb[0] = max(rb[0], max_i |b_i| / ||a_i||^2) and
+// fused pass over the rows [r0, r1) of one block: validation of columns (against [0, nvox)),
+// values and b (flags 4 / 8 / 16), inv_norm2 of the rows and the block's hit counts: cnt[j] += 1,
+// or with cs (FP32 path) cs[j] += {1, |a_ij|}, rb[0] = max(rb[0], max_i |b_i| / ||a_i||^2) and
 // rb[1] = max(rb[1], max |a_ij|).  col and val hold the entries from e0 on: entry p is
-// col[p - e0] (0 for whole arrays, the block's first entry for a staging slot).
+// col[p - e0] (0 for whole arrays, the block's first entry for a staging slot).  With ent (FP32
+// values in CSR32 storage) col is canonical and entry p is also packed into pair p of ent, its
+// column in the order of vm; without it col is in that order already.
 cudaError_t k_prep_block(const int64_t* row_ptr, const int32_t* col, const void* val, int64_t e0, int vdt,
-                         const void* b, int64_t r0, int64_t r1, int64_t nvox, void* inv_norm2, int cdt, int32_t* cnt,
-                         int* flags, float* colsum, float* rb, cudaStream_t s);
-// *out = max(*out, max_j v[j]) for n non-negative floats
-cudaError_t k_colmax(const float* v, int64_t n, float* out, cudaStream_t s);
+                         const void* b, int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inv_norm2,
+                         int cdt, int32_t* cnt, int* flags, float2* cs, float* rb, int32_t* ent, cudaStream_t s);
+// inv_s = 1 / hit count from cs, *lmax = max(*lmax, largest column sum), cs cleared;
+// flags |= 64 when a count reached 2^24 (recount then)
+cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, float* lmax, int* flags, cudaStream_t s);
+// cnt[j] += hits of the packed entries of rows [r0, r1)
+cudaError_t k_recount(const int64_t* row_ptr, int64_t r0, int64_t r1, const int32_t* ent, int32_t* cnt, cudaStream_t s);
 // col_out[p] = internal index of voxel col_in[p]; flags |= 4 for a column outside [0, V)
 // (written as 0).  col_in == col_out is allowed.
 cudaError_t k_remap_cols(const int32_t* col_in, int32_t* col_out, int64_t nnz, VoxMap m, int* flags, cudaStream_t s);
@@ -191,7 +196,6 @@ struct DropSegment {
 // (packed_entries) reads pairs.
 template <typename V, bool D16>
 __host__ __device__ constexpr bool packed_entries() { return !D16 && std::is_same<V, float>::value; }
-cudaError_t k_pack_entries(const int32_t* col, const float* val, int64_t n, int32_t* ent, cudaStream_t s);
 
 struct DropArgs {
     const int64_t* row_ptr;
