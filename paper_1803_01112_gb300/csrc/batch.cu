@@ -5,7 +5,7 @@
 //
 // Work model.  A member's cycle is a sequence of phases,
 //     [GRAD(n), (TRY(n) ...), APPLY(n)] for n < N,  [DROP(b), DAPPLY(b)] for b < B,  PHI,
-// each cut into items: runs of kTvItem voxels (GRAD, TRY, APPLY, DAPPLY, PHI) or of a
+// each cut into items: runs of at most kTvItem voxels (GRAD, TRY, APPLY, DAPPLY, PHI) or of a
 // member-specific number of rows of block b (DROP).  Phases of one member run in order;
 // phases of different members overlap.  Every member has a 64-bit word (phase epoch |
 // items in the phase | cursor); a CTA takes an item with one atomic add on the cursor,
@@ -51,7 +51,7 @@ namespace ntvs {
 namespace {
 
 constexpr int kThreads = 256;     // threads per CTA of the persistent kernel
-constexpr int kTvItem = 2048;     // voxels per voxel item (256 threads x 8)
+constexpr int kTvItem = 2048;     // most voxels of a voxel item (256 threads x 8); fewer in small batches
 constexpr int kSpec = 4;          // TV-check tries evaluated per pass
 constexpr int kBetaTab = 4096;    // beta0 alpha^ell from the host for ell < kBetaTab
 constexpr unsigned long long kM24 = 0xffffffull;
@@ -89,7 +89,7 @@ struct MemberDev {
     double beta0, alpha;
     int check, max_retries, rule;
     uint64_t seed;
-    int lpr, rows_per_item, n_vox_items, part_off;
+    int lpr, rows_per_item, vox_item, n_vox_items, part_off;
 };
 
 // Mutable per-member state of the schedule.
@@ -144,7 +144,7 @@ __device__ __forceinline__ double ordered_sum(const double* a, int n, int stride
 __device__ void grad_item(const MemberDev& m, int idx, double* part, double* part2, double* sh) {
     const int nx = m.nx, ny = m.ny, nz = m.nz;
     const int64_t sxy = (int64_t)nx * ny;
-    const int64_t i0 = (int64_t)idx * kTvItem, i1 = min(m.V, i0 + kTvItem);
+    const int64_t i0 = (int64_t)idx * m.vox_item, i1 = min(m.V, i0 + m.vox_item);
     const float* xh = m.xh;
     const float* xl = m.xl;
     const float eps = m.eps;
@@ -202,7 +202,7 @@ __device__ __forceinline__ double beta_of(const MemberDev& m, int64_t ell) {
 __device__ void try_item(const MemberDev& m, int idx, int64_t ell, int T, double gnorm2, double* part_try, double* sh) {
     const int nx = m.nx, ny = m.ny, nz = m.nz;
     const int64_t sxy = (int64_t)nx * ny;
-    const int64_t i0 = (int64_t)idx * kTvItem, i1 = min(m.V, i0 + kTvItem);
+    const int64_t i0 = (int64_t)idx * m.vox_item, i1 = min(m.V, i0 + m.vox_item);
     double sc[kSpec], acc[kSpec];
 #pragma unroll
     for (int t = 0; t < kSpec; ++t) {
@@ -239,7 +239,7 @@ __device__ void try_item(const MemberDev& m, int idx, int64_t ell, int T, double
 
 // x <- x - sc g on the item's voxels, and the FP32 copies
 __device__ void apply_item(const MemberDev& m, int idx, double sc) {
-    const int64_t i0 = (int64_t)idx * kTvItem, i1 = min(m.V, i0 + kTvItem);
+    const int64_t i0 = (int64_t)idx * m.vox_item, i1 = min(m.V, i0 + m.vox_item);
     for (int64_t p = i0 + threadIdx.x; p < i1; p += blockDim.x) {
         const double z = perturbed(m.x[p], sc, (double)m.g[p]);
         m.x[p] = z;
@@ -253,7 +253,7 @@ __device__ void apply_item(const MemberDev& m, int idx, double sc) {
 // x += delta / s for block b on the item's voxels; delta cleared; after the last block
 // also xh, xl (read by the next cycle's gradient only)
 __device__ void dapply_item(const MemberDev& m, int idx, int b) {
-    const int64_t i0 = (int64_t)idx * kTvItem, i1 = min(m.V, i0 + kTvItem);
+    const int64_t i0 = (int64_t)idx * m.vox_item, i1 = min(m.V, i0 + m.vox_item);
     const float* inv_s = m.inv_s + (int64_t)b * m.vm.vint;
     const bool last = b == m.B - 1;
     for (int64_t j = i0 + threadIdx.x; j < i1; j += blockDim.x) {
@@ -274,7 +274,7 @@ __device__ void dapply_item(const MemberDev& m, int idx, int b) {
 __device__ void phi_item(const MemberDev& m, int idx, double* part, double* sh) {
     const int nx = m.nx, ny = m.ny, nz = m.nz;
     const int64_t sxy = (int64_t)nx * ny;
-    const int64_t i0 = (int64_t)idx * kTvItem, i1 = min(m.V, i0 + kTvItem);
+    const int64_t i0 = (int64_t)idx * m.vox_item, i1 = min(m.V, i0 + m.vox_item);
     double acc = 0.0;
     for (int64_t p = i0 + threadIdx.x; p < i1; p += blockDim.x) {
         int ix, iy, iz;
@@ -307,7 +307,13 @@ __device__ void drop_rows(const MemberDev& m, int64_t i0, int64_t i1, int w0, in
         const int64_t i = base + lane / LPR;
         const bool valid = i < i1;
         int64_t p0 = 0, p1 = 0;
-        if (valid) { p0 = __ldg(m.row_ptr + i); p1 = __ldg(m.row_ptr + i + 1); }
+        float bi = 0.f, ii = 0.f;   // with the extent: after the dot product they would be one more round trip
+        if (valid) {
+            p0 = __ldg(m.row_ptr + i);
+            p1 = __ldg(m.row_ptr + i + 1);
+            bi = __ldg(m.b + i);
+            ii = __ldg(m.inv_norm2 + i);
+        }
         int32_t c[CH];
         float a[CH];
 #pragma unroll
@@ -335,8 +341,8 @@ __device__ void drop_rows(const MemberDev& m, int64_t i0, int64_t i1, int w0, in
         for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         float r = 0.f, rn = 0.f;
         if (valid) {
-            const float res = __ldg(m.b + i) - acc;
-            rn = res * __ldg(m.inv_norm2 + i);
+            const float res = bi - acc;
+            rn = res * ii;
             r = m.lambda * rn;
             if (sub == 0) ss += (double)res * (double)res;
             // the block's largest |r / lambda| (the next sweep's window bound); a plain read
@@ -402,10 +408,6 @@ __device__ void drop_item(const MemberDev& m, int b, int idx, int win_cap, doubl
             bnd = fminf(bound, 0x1p22f * Q / (lam * amax));
         }
     }
-    if (w0 >= 0) {
-        for (int j = threadIdx.x; j < win_cap; j += blockDim.x) batch_win[j] = 0.f;   // int 0 has the bits of 0.0f
-        __syncthreads();
-    }
     switch (m.lpr) {
         case 8: drop_rows<8, 16>(m, r0, r1, w0, win_cap, m.resid + b, sh, invQ, bnd, obs); break;
         case 16: drop_rows<16, 10>(m, r0, r1, w0, win_cap, m.resid + b, sh, invQ, bnd, obs); break;
@@ -414,10 +416,13 @@ __device__ void drop_item(const MemberDev& m, int b, int idx, int win_cap, doubl
     if (w0 >= 0) {
         __syncthreads();
         const int64_t n = min((int64_t)win_cap, m.vm.vint - (int64_t)w0);
-        const int* wint = reinterpret_cast<const int*>(batch_win);
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        int* wint = reinterpret_cast<int*>(batch_win);
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {   // the window is zero again afterwards
             const int v = wint[j];
-            if (v != 0) atomicAdd(m.delta + w0 + j, (float)v * Q);
+            if (v != 0) {
+                atomicAdd(m.delta + w0 + j, (float)v * Q);
+                wint[j] = 0;
+            }
         }
     }
 }
@@ -578,6 +583,7 @@ __global__ void __launch_bounds__(kThreads, MINB) batch_cycle_kernel(CycleArgs a
     const int lane = threadIdx.x & 31;
     int start = blockIdx.x % a.R;
     uint64_t idle0 = 0;
+    for (int j = threadIdx.x; j < a.win_cap; j += blockDim.x) batch_win[j] = 0.f;   // int 0 has the bits of 0.0f
     for (;;) {
         if (threadIdx.x < 32) {   // warp 0 looks for an item, 32 members per probe
             int got = -1, gidx = 0, gitems = 0;
@@ -945,6 +951,8 @@ struct ntvs_batch {
     double* part2 = nullptr;
     double* part_try = nullptr;
     double* beta = nullptr;          // [N_max][R]
+    float* stage = nullptr;          // FP32 image on its way to the host (the largest one asked for)
+    size_t stage_bytes = 0;
     double* hbeta[2] = {nullptr, nullptr};
     int N_max = 0;
     int total_vox_items = 0;
@@ -1283,6 +1291,7 @@ int ntvs_batch_destroy(ntvs_batch* bt) {
     cudaFree(bt->part2);
     cudaFree(bt->part_try);
     cudaFree(bt->beta);
+    cudaFree(bt->stage);
     for (int j = 0; j < 2; ++j) {
         if (bt->hbeta[j]) cudaFreeHost(bt->hbeta[j]);
         if (bt->graph[j]) cudaGraphExecDestroy(bt->graph[j]);
@@ -1494,9 +1503,19 @@ int ntvs_batch_finalize(ntvs_batch* bt, int max_cycles) {
     bt->tv_cap = max_cycles;
     bt->N_max = 0;
     int off = 0;
+    int sms = 0;
+    BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device));
+    // voxels per item: a member's voxel phases are part of its serial chain, so a small batch cuts
+    // them finer, until all members together have three items per resident CTA (16 members of
+    // 64..128 voxels a side: 4.38 -> 4.02 ms per cycle with the finer row items)
+    int64_t all_vox = 0;
+    for (const auto& mm : bt->m) all_vox += mm.d.V;
+    int vox_item = kTvItem;
+    while (vox_item > 512 && all_vox / vox_item < (int64_t)sms * 12) vox_item /= 2;
     for (auto& mm : bt->m) {
         MemberDev& d = mm.d;
-        d.n_vox_items = (int)((d.V + kTvItem - 1) / kTvItem);
+        d.vox_item = vox_item;
+        d.n_vox_items = (int)((d.V + vox_item - 1) / vox_item);
         if ((int64_t)d.n_vox_items > (int64_t)(kM24 >> 1)) return bfail(NTVS_ERR_ARG, "member too large");
         d.part_off = off;
         off += d.n_vox_items;
@@ -1524,8 +1543,6 @@ int ntvs_batch_finalize(ntvs_batch* bt, int max_cycles) {
         std::memset(bt->hbeta[j], 0, sizeof(double) * std::max(bt->N_max, 1) * R);
         BCUDA(cudaEventCreateWithFlags(&bt->used[j], cudaEventDisableTiming));
     }
-    int sms = 0;
-    BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bt->device));
     BCUDA(cudaFuncSetAttribute(batch_cycle_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152 * 4));
     BCUDA(cudaFuncSetAttribute(batch_cycle_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152 * 4));
     auto set_grid = [&](int cap, int minb) -> int {
@@ -1541,7 +1558,15 @@ int ntvs_batch_finalize(ntvs_batch* bt, int max_cycles) {
     };
     // schedule: fixed by the caller, else timed over kTrialCycles cycles per candidate
     // (images and schedule state saved before and restored after)
-    std::vector<int> rows_c = bt->req_rows > 0 ? std::vector<int>{bt->req_rows} : std::vector<int>{256, 512, 1024};
+    // rows per item: three sizes by the rows that a DROP phase of every member has per resident
+    // CTA; small members need small items to keep the CTAs busy (BATCH_NOTE)
+    int64_t phase_rows = 0;
+    for (const auto& mm : bt->m) phase_rows += mm.M / std::max<int64_t>(1, (int64_t)mm.block_ptr.size() - 1);
+    const int64_t per_cta = phase_rows / std::max(1, sms * 4);
+    std::vector<int> rows_c = bt->req_rows > 0  ? std::vector<int>{bt->req_rows}
+                              : per_cta >= 1024 ? std::vector<int>{256, 512, 1024}
+                              : per_cta >= 256  ? std::vector<int>{128, 256, 512}
+                                                : std::vector<int>{64, 128, 256};
     std::vector<int> win_c = bt->req_win >= 0 ? std::vector<int>{bt->req_win} : std::vector<int>{0, 8192, 12288, 16384};
     std::vector<int> minb_c = (bt->req_rows > 0 && bt->req_win >= 0) ? std::vector<int>{3} : std::vector<int>{3, 4};
     if (rows_c.size() * win_c.size() * minb_c.size() == 1) {
@@ -1697,20 +1722,24 @@ int ntvs_batch_get_image(ntvs_batch* bt, int index, void* out, int dtype, int me
     if (mem_kind != NTVS_MEM_HOST && mem_kind != NTVS_MEM_DEVICE) return bfail(NTVS_ERR_ARG, "bad mem_kind");
     BTRY(ntvs_batch_sync(bt));
     const MemberDev& d = bt->m[index].d;
-    std::vector<double> x((size_t)d.V);
-    BCUDA(cudaMemcpy(x.data(), d.x, sizeof(double) * d.V, cudaMemcpyDeviceToHost));
-    if (mem_kind == NTVS_MEM_HOST) {
-        if (dtype == NTVS_F64) std::memcpy(out, x.data(), sizeof(double) * d.V);
-        else for (int64_t j = 0; j < d.V; ++j) ((float*)out)[j] = (float)x[j];
-        return NTVS_OK;
-    }
-    if (dtype == NTVS_F64) {
-        BCUDA(cudaMemcpy(out, x.data(), sizeof(double) * d.V, cudaMemcpyHostToDevice));
+    // converted on the device, straight into a device output or through a buffer of the batch
+    const size_t bytes = (dtype == NTVS_F64 ? sizeof(double) : sizeof(float)) * (size_t)d.V;
+    if (mem_kind == NTVS_MEM_DEVICE) {
+        BCUDA(k_convert(d.x, F64, out, dtype, d.V, bt->stream));
+    } else if (dtype == NTVS_F64) {
+        BCUDA(cudaMemcpyAsync(out, d.x, bytes, cudaMemcpyDeviceToHost, bt->stream));
     } else {
-        std::vector<float> f((size_t)d.V);
-        for (int64_t j = 0; j < d.V; ++j) f[j] = (float)x[j];
-        BCUDA(cudaMemcpy(out, f.data(), sizeof(float) * d.V, cudaMemcpyHostToDevice));
+        if (bt->stage_bytes < bytes) {
+            cudaFree(bt->stage);
+            bt->stage = nullptr;
+            bt->stage_bytes = 0;
+            BTRY(balloc(&bt->stage, bytes, "image read-back"));
+            bt->stage_bytes = bytes;
+        }
+        BCUDA(k_convert(d.x, F64, bt->stage, F32, d.V, bt->stream));
+        BCUDA(cudaMemcpyAsync(out, bt->stage, bytes, cudaMemcpyDeviceToHost, bt->stream));
     }
+    BCUDA(cudaStreamSynchronize(bt->stream));
     return NTVS_OK;
 }
 
