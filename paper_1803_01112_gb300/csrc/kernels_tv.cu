@@ -15,40 +15,42 @@ int red_grid(int64_t n, int sm_count) {
     return (int)(need < cap ? need : cap);
 }
 
-// n / D for several n and one D: 1/D once, every product n (1/D) corrected by its residual
-// (Markstein 1990), 3 FP64 operations a quotient after the first instead of a whole division.
-// D outside the range where the residual is exact divides.
+// n / D for several n and D = sqrt(s): every product n (1/D) corrected by its residual
+// (Markstein 1990), 3 FP64 operations a quotient instead of a division.  D outside the range
+// where the residual is exact divides.
 struct Quotients {
     double D, r;
-    bool safe, some;
-    __device__ __forceinline__ explicit Quotients(double d) : D(d) {
-        const int e = __double2hiint(d);   // 2^-400 < D < 2^400
+    bool safe;
+    __device__ __forceinline__ explicit Quotients(double s) {
+        D = sqrt_and_inverse(s, &r);
+        const int e = __double2hiint(D);   // 2^-400 < D < 2^400
         safe = e > 0x26f00000 && e < 0x58f00000;
-        some = d > 0.0;
-        r = some ? 1.0 / d : 0.0;
     }
     __device__ __forceinline__ double operator()(double n) const {
-        if (!some) return 0.0;
-        if (!safe) return n / D;
+        if (!safe) return D > 0.0 ? n / D : 0.0;
         const double q = n * r;
         return fma(fma(-q, D, n), r, q);
     }
 };
 
-// FP64 path: grad phi_eps on 31 x 15 voxel tiles, marching along z:
+// FP64 path: grad phi_eps on tiles of 31 x (TY - 1) voxels, marching along z:
 //   g_q = -sum_a d_a(q) / D_q + sum_{a: q-e_a inside} d_a(q-e_a) / D_{q-e_a}
 // with d_a(c) = x_{c+e_a} - x_c (0 past the last index) and D_c = sqrt(eps + |d(c)|^2).
 // Every voxel of the tile and of its low halo forms its three quotients d_a / D once; the x and
 // y ones go to the next voxels through shared memory, the z one stays in the thread for the
 // next slice.
 // One thread per voxel forming all four D's of its stencil itself spent 4 square roots and 6
-// divisions a voxel on a pipe of 2 lanes per clock and SM: 145 us on 200x200x16, 74 us here.
+// divisions a voxel on a pipe of 2 lanes per clock and SM: 145 us on 200x200x16, 67 us here.
 // The FP32 path is bound by the latency of its loads instead and keeps one thread per voxel
 // (tiles: 7.5 against 5.5 us on 41x37x5, 58 against 59 us on 256x256x64).
 // PHI: also phi_0(x).
-constexpr int kGradTx = 32, kGradTy = 16;   // threads of a tile: its voxels and one low halo row and column
+//
+// TY: threads of a tile in y.  16 where the tiles fill the SMs; an image of few tiles takes 4 (a
+// quarter of the FP64 work on each of four times as many SMs, for a halo of a row in 3): 10.2 us
+// with 16 and 5.5 us with 4 on 32x32x1.
+constexpr int kGradTx = 32;   // threads of a tile in x: its voxels and one low halo column
 
-template <bool PHI>
+template <bool PHI, int kGradTy>
 __global__ void __launch_bounds__(kGradTx * kGradTy)
 tv_grad_tile_kernel(const double* __restrict__ x, double* __restrict__ g, int nx, int ny, int nz, double eps, int zc,
                     int tiles_x, int tiles, int work, double* partials, unsigned* ticket, double* gnorm2,
@@ -78,7 +80,7 @@ tv_grad_tile_kernel(const double* __restrict__ x, double* __restrict__ g, int nx
                 }
             }
             const double d2 = dx * dx + dy * dy + dz * dz;
-            const Quotients over(sqrt(eps + d2));
+            const Quotients over(eps + d2);
             const int buf = z & 1;
             qxs[buf][ty][tx] = over(dx);
             qys[buf][ty][tx] = over(dy);
@@ -106,71 +108,20 @@ tv_grad_tile_kernel(const double* __restrict__ x, double* __restrict__ g, int nx
     }
 }
 
-// One voxel of grad phi_eps:
-//   g_q = -sum_a d_a(q) / D_q + sum_{a: q-e_a inside} d_a(q-e_a) / D_{q-e_a}
-// with d_a(c) = x_{c+e_a} - x_c (0 past the last index) and D_c = sqrt(eps + |d(c)|^2).
-// The image is the FP64 master copy; differences are formed in FP64 (so nearly equal
-// neighbours keep their difference) and the rest of the arithmetic runs in T.
-template <typename T>
+// FP32 path: the gradient from the split copies xh + xl of the master image, one thread per
+// voxel: every neighbour difference is (xh_a - xh_b) + (xl_a - xl_b) in FP32, so the stencil
+// runs without FP64 arithmetic (only ||g||^2 is accumulated in FP64).  PHI: also phi_0(x) from the
+// master image, its three differences and square root being the pass's only FP64 stencil work
+// (with every difference of the gradient taken in FP64 too, 31.7 us on 128x128x16; 29.5 us).
+template <bool PHI>
 __global__ void __launch_bounds__(kRedThreads)
-tv_grad_kernel(const double* __restrict__ x, T* __restrict__ g, int nx, int ny, int nz, T eps,
-               double* partials, unsigned* ticket, double* gnorm2, double* phi) {
-    const int64_t sxy = (int64_t)nx * ny, V = sxy * nz;
-    double acc[2] = {0.0, 0.0};
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < V; p += (int64_t)gridDim.x * blockDim.x) {
-        int ix, iy, iz;
-        voxel_coords(p, nx, ny, ix, iy, iz);
-        const bool hx = ix + 1 < nx, hy = iy + 1 < ny, hz = iz + 1 < nz;
-        const double xc = __ldg(x + p);
-        const double ex = hx ? __ldg(x + p + 1) - xc : 0.0;
-        const double ey = hy ? __ldg(x + p + nx) - xc : 0.0;
-        const double ez = hz ? __ldg(x + p + sxy) - xc : 0.0;
-        const T dx = (T)ex, dy = (T)ey, dz = (T)ez;
-        const T D = sqrt(eps + (dx * dx + dy * dy + dz * dz));
-        T gq = (D > (T)0) ? -(dx + dy + dz) / D : (T)0;
-        if (ix > 0) {
-            const double xm = __ldg(x + p - 1);
-            const T a = (T)(xc - xm);
-            const T b = hy ? (T)(__ldg(x + p - 1 + nx) - xm) : (T)0;
-            const T c = hz ? (T)(__ldg(x + p - 1 + sxy) - xm) : (T)0;
-            const T Dm = sqrt(eps + (a * a + b * b + c * c));
-            if (Dm > (T)0) gq += a / Dm;
-        }
-        if (iy > 0) {
-            const double xm = __ldg(x + p - nx);
-            const T a = (T)(xc - xm);
-            const T b = hx ? (T)(__ldg(x + p - nx + 1) - xm) : (T)0;
-            const T c = hz ? (T)(__ldg(x + p - nx + sxy) - xm) : (T)0;
-            const T Dm = sqrt(eps + (a * a + b * b + c * c));
-            if (Dm > (T)0) gq += a / Dm;
-        }
-        if (iz > 0) {
-            const double xm = __ldg(x + p - sxy);
-            const T a = (T)(xc - xm);
-            const T b = hx ? (T)(__ldg(x + p - sxy + 1) - xm) : (T)0;
-            const T c = hy ? (T)(__ldg(x + p - sxy + nx) - xm) : (T)0;
-            const T Dm = sqrt(eps + (a * a + b * b + c * c));
-            if (Dm > (T)0) gq += a / Dm;
-        }
-        g[p] = gq;
-        acc[0] += (double)gq * (double)gq;
-        if (phi) acc[1] += sqrt(ex * ex + ey * ey + ez * ez);
-    }
-    double* const outs[2] = {gnorm2, phi};
-    grid_reduce<2>(acc, partials, ticket, outs);
-}
-
-// The same gradient on the FP32 path from the split copies xh + xl of the master image:
-// every neighbour difference is (xh_a - xh_b) + (xl_a - xl_b) in FP32, so the stencil runs
-// without FP64 arithmetic (only ||g||^2 is accumulated in FP64).
-__global__ void __launch_bounds__(kRedThreads)
-tv_grad_split_kernel(const float* __restrict__ xh, const float* __restrict__ xl, float* __restrict__ g, int nx,
-                     int ny, int nz, float eps, double* partials, unsigned* ticket, double* gnorm2) {
+tv_grad_split_kernel(const double* __restrict__ x, const float* __restrict__ xh, const float* __restrict__ xl, float* __restrict__ g, int nx,
+                     int ny, int nz, float eps, double* partials, unsigned* ticket, double* gnorm2, double* phi) {
     const int64_t sxy = (int64_t)nx * ny, V = sxy * nz;
     auto dif = [&](int64_t a, int64_t b) -> float {
         return (__ldg(xh + a) - __ldg(xh + b)) + (__ldg(xl + a) - __ldg(xl + b));
     };
-    double acc[1] = {0.0};
+    double acc[PHI ? 2 : 1] = {};
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < V; p += (int64_t)gridDim.x * blockDim.x) {
         int ix, iy, iz;
         voxel_coords(p, nx, ny, ix, iy, iz);
@@ -198,9 +149,20 @@ tv_grad_split_kernel(const float* __restrict__ xh, const float* __restrict__ xl,
         }
         g[p] = gq;
         acc[0] += (double)gq * (double)gq;
+        if constexpr (PHI) {
+            const double xc = __ldg(x + p);
+            const double ex = hx ? __ldg(x + p + 1) - xc : 0.0, ey = hy ? __ldg(x + p + nx) - xc : 0.0,
+                         ez = hz ? __ldg(x + p + sxy) - xc : 0.0;
+            acc[1] += sqrt(ex * ex + ey * ey + ez * ez);
+        }
     }
-    double* const outs[1] = {gnorm2};
-    grid_reduce<1>(acc, partials, ticket, outs);
+    if constexpr (PHI) {
+        double* const outs[2] = {gnorm2, phi};
+        grid_reduce<2>(acc, partials, ticket, outs);
+    } else {
+        double* const outs[1] = {gnorm2};
+        grid_reduce<1>(acc, partials, ticket, outs);
+    }
 }
 
 // phi_0(z), z = x - sc*g (z = x if g is null), FP64 from the master image.
@@ -300,7 +262,7 @@ static int sm_count() {
     return g_sm_count;
 }
 
-template <bool PHI>
+template <bool PHI, int kGradTy>
 static cudaError_t launch_grad_tile(const double* x, double* g, int nx, int ny, int nz, double eps, RedScratch r,
                                     double* gnorm2, double* phi, cudaStream_t s) {
     const int tiles_x = (nx + kGradTx - 2) / (kGradTx - 1), tiles_y = (ny + kGradTy - 2) / (kGradTy - 1);
@@ -318,22 +280,22 @@ static cudaError_t launch_grad_tile(const double* x, double* g, int nx, int ny, 
     }
     const int64_t work = tiles * ((nz + zc - 1) / zc);   // below the voxel count's 2^31
     const int grid = (int)(work < (int64_t)sms * 4 ? work : (int64_t)sms * 4);
-    tv_grad_tile_kernel<PHI><<<grid, kGradTx * kGradTy, 0, s>>>(x, g, nx, ny, nz, eps, zc, tiles_x, (int)tiles,
+    tv_grad_tile_kernel<PHI, kGradTy><<<grid, kGradTx * kGradTy, 0, s>>>(x, g, nx, ny, nz, eps, zc, tiles_x, (int)tiles,
                                                                (int)work, r.partials, r.ticket, gnorm2, phi);
     return cudaGetLastError();
 }
 
 cudaError_t k_tv_grad(int cdt, const double* x, const float* xh, const float* xl, void* g, int nx, int ny, int nz,
                       double eps, RedScratch r, double* gnorm2, double* phi, cudaStream_t s) {
-    if (cdt == F64)
-        return phi ? launch_grad_tile<true>(x, (double*)g, nx, ny, nz, eps, r, gnorm2, phi, s)
-                   : launch_grad_tile<false>(x, (double*)g, nx, ny, nz, eps, r, gnorm2, phi, s);
-    if (xh && xl && !phi)
-        tv_grad_split_kernel<<<r.grid, kRedThreads, 0, s>>>(xh, xl, (float*)g, nx, ny, nz, (float)eps, r.partials,
-                                                           r.ticket, gnorm2);
-    else
-        tv_grad_kernel<float><<<r.grid, kRedThreads, 0, s>>>(x, (float*)g, nx, ny, nz, (float)eps, r.partials,
-                                                             r.ticket, gnorm2, phi);
+    if (cdt == F64) {
+        const bool few = (int64_t)nx * ny * nz < (int64_t)sm_count() * kGradTx * 16;   // under a tile slice an SM
+        const auto run = few ? (phi ? launch_grad_tile<true, 4> : launch_grad_tile<false, 4>)
+                             : (phi ? launch_grad_tile<true, 16> : launch_grad_tile<false, 16>);
+        return run(x, (double*)g, nx, ny, nz, eps, r, gnorm2, phi, s);
+    }
+    if (!xh || !xl) return cudaErrorInvalidValue;   // the FP32 path keeps the split copies
+    (phi ? tv_grad_split_kernel<true> : tv_grad_split_kernel<false>)<<<r.grid, kRedThreads, 0, s>>>(
+        x, xh, xl, (float*)g, nx, ny, nz, (float)eps, r.partials, r.ticket, gnorm2, phi);
     return cudaGetLastError();
 }
 
