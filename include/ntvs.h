@@ -95,7 +95,9 @@ typedef struct {
  * with the matrix streamed into shared memory by the TMA engine (cp.async.bulk) ahead of
  * the consumer warps; needs 16-byte aligned col/val and 64 KB more shared memory.  When
  * the slice fits and rows come in runs of the same slice (e.g. stored by projection angle,
- * then slice), AUTO picks WINDOW (measured fastest); otherwise PLAIN.  With FP64
+ * then slice), AUTO picks WINDOW (measured fastest); otherwise PLAIN,
+ * except that large blocks of FP32 rows stored in another order are grouped by slice for
+ * WINDOW (an index of the rows; the stored order stays).  With FP64
  * arithmetic WINDOW keeps no window and scatters with global reductions (measured faster).  Every schedule reads
  * both index storages.  All give the same result up to the order of floating-point
  * summation. */

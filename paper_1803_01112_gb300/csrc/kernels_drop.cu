@@ -239,7 +239,8 @@ cudaError_t k_row_home(const int64_t* row_ptr, const int32_t* col, int stride, i
 
 // A warp per chunk of rows: the chunk's work in issued register steps (k_chunk_cost); a
 // chunk of a block without a per-block depth (ch = 0) counts its rows
-__global__ void chunk_cost_kernel(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ cs,
+__global__ void chunk_cost_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ order,
+                                  const int64_t* __restrict__ cs,
                                   const int8_t* __restrict__ ch, int mid, int64_t nchunks, int64_t* __restrict__ cost) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -253,7 +254,8 @@ __global__ void chunk_cost_kernel(const int64_t* __restrict__ row_ptr, const int
                 acc += 4;
                 continue;
             }
-            const int64_t steps = (row_ptr[i + 1] - row_ptr[i] + 31) / 32;
+            const int64_t row = order ? order[i] : i;
+            const int64_t steps = (row_ptr[row + 1] - row_ptr[row] + 31) / 32;
             const int64_t body = (steps <= kShortBody && d > kShortBody) ? kShortBody
                                  : (mid > 0 && d > mid && steps <= mid) ? mid : d;
             const int64_t live = steps < body ? steps : body;
@@ -264,10 +266,69 @@ __global__ void chunk_cost_kernel(const int64_t* __restrict__ row_ptr, const int
     }
 }
 
-cudaError_t k_chunk_cost(const int64_t* row_ptr, const int64_t* cs, const int8_t* ch, int mid, int64_t nchunks,
-                         int64_t* cost, int grid, cudaStream_t s) {
+cudaError_t k_chunk_cost(const int64_t* row_ptr, const int32_t* order, const int64_t* cs, const int8_t* ch, int mid,
+                         int64_t nchunks, int64_t* cost, int grid, cudaStream_t s) {
     if (nchunks <= 0) return cudaSuccess;
-    chunk_cost_kernel<<<grid, 256, 0, s>>>(row_ptr, cs, ch, mid, nchunks, cost);
+    chunk_cost_kernel<<<grid, 256, 0, s>>>(row_ptr, order, cs, ch, mid, nchunks, cost);
+    return cudaGetLastError();
+}
+
+// A CTA per block: a stable counting sort of the block's rows by home slice.  Rows go through in
+// tiles of 1024 in stored order; a row's place is its home's running count, plus the tile's rows
+// of that home in earlier warps, plus those in earlier lanes of its warp.
+__global__ void __launch_bounds__(1024) order_rows_kernel(const int32_t* __restrict__ home,
+                                                          const int64_t* __restrict__ bp, int homes,
+                                                          int32_t* __restrict__ order,
+                                                          int32_t* __restrict__ home_sorted) {
+    extern __shared__ int order_smem[];
+    int* next = order_smem;          // [homes] first free place of each home
+    int* cnt = order_smem + homes;   // [32][homes] a tile's rows of each home per warp
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t r0 = bp[blockIdx.x], r1 = bp[blockIdx.x + 1];
+    for (int h = tid; h < homes; h += 1024) next[h] = 0;
+    __syncthreads();
+    for (int64_t i = r0 + tid; i < r1; i += 1024) atomicAdd(next + min(max(home[i], 0), homes - 1), 1);
+    __syncthreads();
+    if (tid == 0) {
+        int sum = 0;
+        for (int h = 0; h < homes; ++h) {
+            const int n = next[h];
+            next[h] = sum;
+            sum += n;
+        }
+    }
+    for (int64_t t0 = r0; t0 < r1; t0 += 1024) {
+        for (int q = tid; q < 32 * homes; q += 1024) cnt[q] = 0;
+        __syncthreads();
+        const int64_t i = t0 + tid;
+        const int h = i < r1 ? min(max(home[i], 0), homes - 1) : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, h);
+        const int rank = __popc(same & ((1u << lane) - 1u));
+        if (h >= 0 && rank == 0) cnt[warp * homes + h] = __popc(same);
+        __syncthreads();
+        for (int q = tid; q < homes; q += 1024) {
+            int at = next[q];
+            for (int w = 0; w < 32; ++w) {
+                const int n = cnt[w * homes + q];
+                cnt[w * homes + q] = at;
+                at += n;
+            }
+            next[q] = at;
+        }
+        __syncthreads();
+        if (h >= 0) {
+            const int64_t q = r0 + cnt[warp * homes + h] + rank;
+            order[q] = (int32_t)i;
+            home_sorted[q] = h;
+        }
+        __syncthreads();
+    }
+}
+
+cudaError_t k_order_rows(const int32_t* home, const int64_t* bp, int B, int homes, int32_t* order,
+                         int32_t* home_sorted, cudaStream_t s) {
+    if (B <= 0) return cudaSuccess;
+    order_rows_kernel<<<B, 1024, sizeof(int) * 33 * (size_t)homes, s>>>(home, bp, homes, order, home_sorted);
     return cudaGetLastError();
 }
 

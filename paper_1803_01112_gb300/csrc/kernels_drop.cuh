@@ -54,6 +54,13 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&o)[4]) {
 extern __shared__ __align__(16) unsigned char drop_win_smem[];
 template <bool D16>
 __host__ __device__ constexpr int row_stage() { return D16 ? 1600 : 2048; }   // rows staged at once
+// Rows taken through an order (row_order below) stage their starts and lengths instead of the
+// row pointers, 20 bytes a row, in the same space, so that the window stays where it is.
+constexpr int kOrderedStage = 1600;
+__device__ __forceinline__ int64_t* ordered_start() { return reinterpret_cast<int64_t*>(drop_win_smem); }
+__device__ __forceinline__ int32_t* ordered_len() { return reinterpret_cast<int32_t*>(drop_win_smem + 8 * kOrderedStage); }
+__device__ __forceinline__ float* ordered_b() { return reinterpret_cast<float*>(drop_win_smem + 12 * kOrderedStage); }
+__device__ __forceinline__ float* ordered_inv() { return reinterpret_cast<float*>(drop_win_smem + 16 * kOrderedStage); }
 constexpr int kPrefetchRows = 1;  // the windowed kernel asks L2 for the entries of the row this many ahead
 constexpr int kShortSteps = kShortBody;   // register steps of the windowed kernel's body for short rows
 
@@ -436,14 +443,20 @@ __device__ __forceinline__ void flush_window(int* win, int W, float* delta, int 
     }
 }
 
-template <typename T, typename V, int LPR, int CH, int VW, bool D16>
+// ORD (packed pairs): segments are runs of positions in row_order, which groups a block's rows by
+// home slice where they are stored in another order (histories as detected).  A row's entries lie
+// together wherever the row does, so only the staging goes through the order.
+template <typename T, typename V, int LPR, int CH, int VW, bool D16, bool ORD>
 __global__ void __launch_bounds__(1024, 1)
 drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                          const V* __restrict__ val, const T* __restrict__ b, const T* __restrict__ inv_norm2,
                          const DropSegment* __restrict__ segs, const int32_t* __restrict__ seg_begin,
                          int64_t slice, const T* __restrict__ x, T* __restrict__ delta, T lambda,
                          double* resid_ss, Delta16 d16, const float* wlmax, const float* wbound, float* wobs,
-                         const float* wamax) {
+                         const float* wamax, const int32_t* __restrict__ row_order) {
+    static_assert(!ORD || (!D16 && sizeof(T) == 4 && 20 * kOrderedStage <= stage_bytes_all<float, false>()),
+                  "ordered rows are packed FP32 pairs and stage in the space of the others");
+    constexpr int RS = ORD ? kOrderedStage : row_stage<D16>();
     int* win = reinterpret_cast<int*>(window_base<T, D16>());
     const int W = (int)slice;
     __shared__ WinScale ws;
@@ -484,10 +497,18 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
         // the segment's rows in runs of row_stage<D16>(): one coalesced load of their row
         // pointers, b and 1/||a||^2 into shared memory, so that a row starts from its
         // entries' addresses instead of a round trip to HBM for its row pointer
-        for (int64_t c0 = sg.r0; c0 < sg.r1; c0 += row_stage<D16>()) {
-            const int n = (int)min((int64_t)row_stage<D16>(), sg.r1 - c0);
+        for (int64_t c0 = sg.r0; c0 < sg.r1; c0 += RS) {
+            const int n = (int)min((int64_t)RS, sg.r1 - c0);
             __syncthreads();   // the previous run's rows are done with the stage
-            for (int j = threadIdx.x; j <= n; j += blockDim.x) {
+            for (int j = threadIdx.x; ORD && j < n; j += blockDim.x) {
+                const int32_t i = __ldg(row_order + c0 + j);
+                const int64_t q0 = __ldg(row_ptr + i);
+                ordered_start()[j] = q0;
+                ordered_len()[j] = (int32_t)(__ldg(row_ptr + i + 1) - q0);
+                ordered_b()[j] = (float)__ldg(b + i);
+                ordered_inv()[j] = (float)__ldg(inv_norm2 + i);
+            }
+            for (int j = threadIdx.x; !ORD && j <= n; j += blockDim.x) {
                 const int64_t rp = __ldg(row_ptr + c0 + j);
                 stage_rp<T, D16>()[j] = rp;
                 if (j < n) {
@@ -507,7 +528,8 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
                     const int kp = k + kPrefetchRows * nwarps * G;   // this group's row that many iterations ahead
                     const int sub = lane % LPR;
                     if (kp < n) {
-                        const int64_t q0 = stage_rp<T, D16>()[kp], q1 = stage_rp<T, D16>()[kp + 1];
+                        const int64_t q0 = ORD ? ordered_start()[kp] : stage_rp<T, D16>()[kp];
+                        const int64_t q1 = ORD ? q0 + ordered_len()[kp] : stage_rp<T, D16>()[kp + 1];
                         if constexpr (D16) {
                             if constexpr (delta16_words<V, D16>()) prefetch_lines_l2(d16.word, q0, q1, sub);
                             else prefetch_row_l2(d16.off, val, q0, q1, sub);
@@ -521,10 +543,16 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
                         }
                     }
                 }
-                const RowHead h{valid ? stage_rp<T, D16>()[k] : 0, valid ? stage_rp<T, D16>()[k + 1] : 0};
+                RowHead h{0, 0};
+                T bk = (T)0, ik = (T)0;
+                if (valid) {
+                    h.p0 = ORD ? ordered_start()[k] : stage_rp<T, D16>()[k];
+                    h.p1 = ORD ? h.p0 + ordered_len()[k] : stage_rp<T, D16>()[k + 1];
+                    bk = ORD ? (T)ordered_b()[k] : stage_b<T, D16>()[k];
+                    ik = ORD ? (T)ordered_inv()[k] : stage_inv<T, D16>()[k];
+                }
                 drop_row_any<T, V, LPR, CH, VW, true, D16>(
-                    c0 + k, h, valid, lane % LPR, col, d16, val, valid ? stage_b<T, D16>()[k] : (T)0,
-                    valid ? stage_inv<T, D16>()[k] : (T)0, x, delta, lambda, w, ss_grp[warp][grp], &ws,
+                    c0 + k, h, valid, lane % LPR, col, d16, val, bk, ik, x, delta, lambda, w, ss_grp[warp][grp], &ws,
                     D16 ? (valid ? (int)stage_fl<T, D16>()[k] : 0) : -1, (D16 && valid) ? stage_rb<T, D16>()[k] : 0);
             }
         }
@@ -541,22 +569,26 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
 }
 
 // ------------------------------------------------------------------ launch
-template <typename T, typename V, int LPR, int CH, int VW, bool D16>
+template <typename T, typename V, int LPR, int CH, int VW, bool D16, bool ORD>
 cudaError_t launch_window(const DropArgs& a, cudaStream_t s) {
-    auto kern = drop_block_window_kernel<T, V, LPR, CH, VW, D16>;
+    auto kern = drop_block_window_kernel<T, V, LPR, CH, VW, D16, ORD>;
     const size_t smem = window_smem_bytes(a.slice, sizeof(T), D16);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<a.grid, 1024, smem, s>>>(a.row_ptr, a.col, (const V*)a.val, (const T*)a.b, (const T*)a.inv_norm2, a.segs,
                                     a.seg_begin, a.slice, (const T*)a.x, (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16,
-                                    a.wlmax, a.wbound, a.wobs, a.wamax);
+                                    a.wlmax, a.wbound, a.wobs, a.wamax, a.order);
     return cudaGetLastError();
 }
 
 template <typename T, typename V, int LPR, int CH, int VW, bool D16>
 static cudaError_t launch_cfg(const DropArgs& a, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
-        if (a.segs) return launch_window<T, V, LPR, CH, VW, D16>(a, s);
+        if constexpr (packed_entries<V, D16>() && LPR >= 16) {
+            if (a.segs && a.order) return launch_window<T, V, LPR, CH, VW, D16, true>(a, s);
+        }
+        if (a.segs && a.order) return cudaErrorInvalidValue;   // the planner orders packed rows only
+        if (a.segs) return launch_window<T, V, LPR, CH, VW, D16, false>(a, s);
     }
     // no more CTAs than the rows fill (8 warps of 32 / LPR rows each): on 2000 rows of the 32x32
     // slice the 1216 CTAs of a large block, nearly all without a row, took 8.5 us against 5.3

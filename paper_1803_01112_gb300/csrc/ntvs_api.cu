@@ -111,6 +111,7 @@ struct ntvs_ctx {
     int schedule = NTVS_SCHED_PLAIN;
     DropSegment* segs = nullptr;       // windowed schedule: all blocks' segments
     int32_t* seg_begin = nullptr;      // [B][win_grid + 1]
+    int32_t* order = nullptr;          // [M] rows grouped by home slice inside each block (else stored order)
     DropStage* stages = nullptr;       // pipelined schedule: all blocks' stages
     int32_t* stage_begin = nullptr;    // [B][win_grid + 1]
     int win_grid = 0;
@@ -215,6 +216,7 @@ struct ntvs_ctx {
         dev_free(inv_s);
         dev_free(segs);
         dev_free(seg_begin);
+        dev_free(order);
         dev_free(wstat);
         dev_free(stages);
         dev_free(stage_begin);
@@ -561,6 +563,7 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
     a.d16 = c->d16();
     a.segs = nullptr;
     a.seg_begin = nullptr;
+    a.order = nullptr;
     a.slice = c->vm.slice_p;
     a.wlmax = nullptr;
     a.wbound = nullptr;
@@ -569,6 +572,7 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
     a.max_row = t < (int)c->block_maxrow.size() ? c->block_maxrow[t] : (int64_t)1 << 40;
     if (whole && c->schedule == NTVS_SCHED_WINDOW && c->segs) {
         a.segs = c->segs;
+        a.order = c->order;
         a.seg_begin = c->seg_begin + (size_t)t * (c->win_grid + 1);
         a.grid = c->win_grid;
         if (c->wstat) {
@@ -729,6 +733,7 @@ static int pack_delta16(ntvs_ctx* c) {
 // past the row's end issues predicated off and counts a quarter of a live one.
 constexpr int kChunkRows = 64;
 constexpr double kMinMeanRun = 8.0;
+constexpr int64_t kOrderEntries = 12000000;   // mean entries per block from which unordered rows are grouped
 
 static int plan_schedule(ntvs_ctx* c, int requested) {
     c->schedule = NTVS_SCHED_PLAIN;
@@ -771,7 +776,8 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
     const size_t o_changes = o_start + up256(sizeof(int64_t) * cstart.size());
     const size_t o_ch = o_changes + up256(sizeof(unsigned long long));
     const size_t o_cost = o_ch + up256(chunk_ch.size());
-    const size_t scratch_bytes = o_cost + up256(sizeof(int64_t) * nchp);
+    const size_t o_bp = o_cost + up256(sizeof(int64_t) * nchp);
+    const size_t scratch_bytes = o_bp + up256(sizeof(int64_t) * ((size_t)c->B + 1));
     char* scratch = nullptr;
     TRY(dev_alloc(&scratch, scratch_bytes, "schedule planning scratch"));
     struct FreeScratch {
@@ -784,6 +790,7 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
     unsigned long long* dchanges = reinterpret_cast<unsigned long long*>(scratch + o_changes);
     int8_t* dch = reinterpret_cast<int8_t*>(scratch + o_ch);
     int64_t* dcost = reinterpret_cast<int64_t*>(scratch + o_cost);
+    int64_t* dbp = reinterpret_cast<int64_t*>(scratch + o_bp);
     std::vector<int32_t> chome((size_t)nch);
     std::vector<int64_t> ccost((size_t)nch);
     unsigned long long changes = 0;
@@ -798,7 +805,7 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
     // the middle body: every CSR32 row, and the narrow DELTA16 rows (90 % of the benchmark's;
     // the others run the block's depth, which the count slightly underestimates)
     const int mid_body = kMidBody;
-    if (e == cudaSuccess) e = k_chunk_cost(c->row_ptr, dstart, dch, mid_body, nch, dcost, c->sms * 8, c->stream);
+    if (e == cudaSuccess) e = k_chunk_cost(c->row_ptr, nullptr, dstart, dch, mid_body, nch, dcost, c->sms * 8, c->stream);
     if (e == cudaSuccess && nch > 0)
         e = cudaMemcpyAsync(chome.data(), dchunk, sizeof(int32_t) * (size_t)nch, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess && nch > 0)
@@ -806,14 +813,37 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(&changes, dchanges, sizeof(changes), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return fail(NTVS_ERR_CUDA, cuda_msg("row home slices", e));
+    // mean run length of equal home slices in stored order
+    const double mean_run = (double)c->M / (double)(changes + 1);
+    if (requested == NTVS_SCHED_AUTO && mean_run < kMinMeanRun) {
+        // Rows in another order (histories as detected): packed FP32 pairs in large blocks are
+        // grouped by home slice for the window, everything else keeps the plain schedule.  us per
+        // block, plain against grouped: 200x200x16, 52.1 / 51.7 at 15M entries a block and 79.8 /
+        // 70.1 at 25M; 128x128x16, 65.7 / 56.2 at 21M; 96x96x12, 55.4 / 46.2 at 16M.
+        if (!c->ent || c->cdt != F32 || c->win_lpr < 16 || c->nz > kOrderHomes || c->M > INT32_MAX ||
+            c->nnz / std::max(c->B, 1) < kOrderEntries)
+            return NTVS_OK;
+        TRY(dev_alloc(&c->order, sizeof(int32_t) * (size_t)c->M, "row order"));
+        int32_t* dsorted = nullptr;
+        TRY(dev_alloc(&dsorted, sizeof(int32_t) * (size_t)c->M, "ordered home slices"));
+        struct FreeSorted {
+            int32_t*& p;
+            ~FreeSorted() { dev_free(p); }
+        } sorted_guard{dsorted};
+        CUDA_TRY(cudaMemcpyAsync(dbp, c->block_ptr.data(), sizeof(int64_t) * ((size_t)c->B + 1), cudaMemcpyHostToDevice,
+                                 c->stream));
+        CUDA_TRY(k_order_rows(dhome, dbp, c->B, c->nz, c->order, dsorted, c->stream));
+        CUDA_TRY(k_chunk_home(dsorted, dstart, nch, dchunk, dchanges, c->sms * 8, c->stream));
+        CUDA_TRY(k_chunk_cost(c->row_ptr, c->order, dstart, dch, mid_body, nch, dcost, c->sms * 8, c->stream));
+        CUDA_TRY(cudaMemcpyAsync(chome.data(), dchunk, sizeof(int32_t) * (size_t)nch, cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(cudaMemcpyAsync(ccost.data(), dcost, sizeof(int64_t) * (size_t)nch, cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+    }
     int32_t last = 0;
     for (auto& h : chome) {   // chunks of empty rows join their predecessor's run
         if (h < 0) h = last;
         last = h;
     }
-    // mean run length of equal home slices in stored order
-    const double mean_run = (double)c->M / (double)(changes + 1);
-    if (requested == NTVS_SCHED_AUTO && mean_run < kMinMeanRun) return NTVS_OK;
 
     // FP64 arithmetic: the windowed schedule runs without the window.  A shared-memory FP64 add
     // is a compare-and-swap loop, a global one is native, and rows in stored order with global

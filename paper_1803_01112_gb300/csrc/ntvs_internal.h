@@ -218,6 +218,7 @@ struct DropArgs {
     // [seg_begin[c], seg_begin[c+1]); shared window of one z-slice (slice = nx*ny voxels)
     const DropSegment* segs;
     const int32_t* seg_begin;
+    const int32_t* order;   // not null: segments are runs of positions in this row order
     int64_t slice;
     // FP32 windowed schedule: the window accumulates in int32 fixed point with quantum
     // Q = |lambda| * bound * lmax / 2^30, where lmax = max_j sum_{i in block} |a_ij| and
@@ -253,8 +254,15 @@ inline int window_register_steps(int64_t max_row, int cdt, int vdt, int lanes_pe
 // that body past the row's end (issued predicated off: no loads, gathers or scatters) + 8
 // per step past ch[q] (the tail loop reads those entries twice).  Charging empty steps a
 // quarter instead of a full step measured 0.2302 -> 0.2281 ms per 500k-row block.
-cudaError_t k_chunk_cost(const int64_t* row_ptr, const int64_t* cs, const int8_t* ch, int mid, int64_t nchunks,
-                         int64_t* cost, int grid, cudaStream_t s);
+// With order not null the chunks are runs of positions in it.
+cudaError_t k_chunk_cost(const int64_t* row_ptr, const int32_t* order, const int64_t* cs, const int8_t* ch, int mid,
+                         int64_t nchunks, int64_t* cost, int grid, cudaStream_t s);
+// order = the rows of each of the B blocks [bp[t], bp[t+1]) grouped by home slice (below
+// kOrderHomes; rows without one first), stored order inside a group; home_sorted[q] = home of
+// row order[q] (0 for none)
+constexpr int kOrderHomes = 256;
+cudaError_t k_order_rows(const int32_t* home, const int64_t* bp, int B, int homes, int32_t* order,
+                         int32_t* home_sorted, cudaStream_t s);
 cudaError_t k_drop_block_d16(const DropArgs& a, cudaStream_t s);   // the same on DELTA16 storage
 // out[i] = <a_i, x> for the M rows (x: compute type, in the order of the stored columns;
 // out: double when out64, else float); a.row_ptr, col / d16, val, vdt, cdt, use_d16 and grid are used
