@@ -820,8 +820,10 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
         // grouped by home slice for the window, everything else keeps the plain schedule.  us per
         // block, plain against grouped: 200x200x16, 52.1 / 51.7 at 15M entries a block and 79.8 /
         // 70.1 at 25M; 128x128x16, 65.7 / 56.2 at 21M; 96x96x12, 55.4 / 46.2 at 16M.
+        int64_t longest = 0;
+        for (int64_t n : c->block_maxrow) longest = std::max(longest, n);
         if (!c->ent || c->cdt != F32 || c->win_lpr < 16 || c->nz > kOrderHomes || c->M > INT32_MAX ||
-            c->nnz / std::max(c->B, 1) < kOrderEntries)
+            longest > INT32_MAX || c->nnz / std::max(c->B, 1) < kOrderEntries)   // 32-bit rows and lengths
             return NTVS_OK;
         TRY(dev_alloc(&c->order, sizeof(int32_t) * (size_t)c->M, "row order"));
         int32_t* dsorted = nullptr;
