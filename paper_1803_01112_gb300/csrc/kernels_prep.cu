@@ -169,8 +169,8 @@ cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, float* lmax, int
     return cudaGetLastError();
 }
 
-// Hit counts of packed or separate entries [q0, q1) in 32-bit integers, for blocks whose float
-// counts were full; entry q's column is col[stride * q] and its value bits (stride 2) beside it
+// Hit counts of the packed entries of rows [r0, r1) in 32-bit integers, for systems whose float
+// counts were full
 __global__ void recount_kernel(const int64_t* __restrict__ row_ptr, int64_t r0, int64_t r1,
                                const int2* __restrict__ ent, int32_t* __restrict__ cnt) {
     const int64_t q0 = row_ptr[r0], q1 = row_ptr[r1];
