@@ -79,8 +79,9 @@ struct MemberDev {
     float* delta;              // internal order
     float* g;                  // canonical order
     double* resid;             // [B]
-    float* wstat;              // [4B] per block: lmax, bound, observed max (float bits), amax (the
-                               // fixed-point DROP window's scale, as in the single-context kernel)
+    WinStat* wstat;            // [B] statistics of the blocks' rows, and
+    float* rms;                // the rms residual of the last swept block (the fixed-point DROP window's
+                               // scale, as in the single-context kernel)
     double* tv_hist;           // [cap]
     int nx, ny, nz, B, N;
     int64_t V;
@@ -297,7 +298,7 @@ extern __shared__ float batch_win[];   // the shared scatter window (win_cap flo
 // others into global delta, else every entry into global delta
 template <int LPR, int CH>
 __device__ void drop_rows(const MemberDev& m, int64_t i0, int64_t i1, int w0, int win_cap, double* resid_b,
-                          double* sh, float invQ, float bnd, unsigned* obs) {
+                          double* sh, float invQ, float bnd) {
     constexpr int G = 32 / LPR;
     const int lane = threadIdx.x & 31, sub = lane % LPR;
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -345,10 +346,6 @@ __device__ void drop_rows(const MemberDev& m, int64_t i0, int64_t i1, int w0, in
             rn = res * ii;
             r = m.lambda * rn;
             if (sub == 0) ss += (double)res * (double)res;
-            // the block's largest |r / lambda| (the next sweep's window bound); a plain read
-            // first skips the atomic for most rows
-            const unsigned arn = __float_as_uint(fabsf(rn));
-            if (sub == 0 && obs && arn > *(volatile unsigned*)obs) atomicMax(obs, arn);
         }
         // a row within the bound adds its terms to the window as int32 multiples of the
         // quantum (every term below 2^22 quanta, every slot below 2^30): r / Q = r * invQ
@@ -393,25 +390,12 @@ __device__ void drop_item(const MemberDev& m, int b, int idx, int win_cap, doubl
     const int64_t r0 = __ldg(m.block_ptr + b) + (int64_t)idx * m.rows_per_item;
     const int64_t r1 = min(__ldg(m.block_ptr + b + 1), r0 + m.rows_per_item);
     const int w0 = win_cap > 0 ? __ldg(m.win_lo + __ldg(m.item0 + b) + idx) : -1;
-    // the window's quantum Q = |lambda| bound lmax / 2^30 from the block's statistics (lmax:
-    // the largest column sum of |a_ij| over the block's rows, so no slot passes 2^30 Q);
-    // rows above min(bound, 2^22 Q / (|lambda| amax)) go to global memory
-    float Q = 0.f, invQ = 0.f, bnd = 0.f;
-    unsigned* obs = m.wstat ? reinterpret_cast<unsigned*>(m.wstat + 2 * m.B + b) : nullptr;
-    if (w0 >= 0 && m.wstat) {
-        const float lmax = m.wstat[b], bound = m.wstat[m.B + b], amax = m.wstat[3 * m.B + b];
-        const float lam = fabsf(m.lambda);
-        Q = lam * bound * lmax * 0x1p-30f;
-        const float iq = 1.f / Q;
-        if (bound > 0.f && amax > 0.f && Q > 0.f && isfinite(Q) && isfinite(iq)) {
-            invQ = iq;
-            bnd = fminf(bound, 0x1p22f * Q / (lam * amax));
-        }
-    }
+    // the rms residual was written by the CTA that finished the block before (in this launch)
+    const WinScale ws = w0 >= 0 ? win_scale(m.lambda, m.wstat[b], *(volatile float*)m.rms) : WinScale{0.f, 0.f, 0.f};
     switch (m.lpr) {
-        case 8: drop_rows<8, 16>(m, r0, r1, w0, win_cap, m.resid + b, sh, invQ, bnd, obs); break;
-        case 16: drop_rows<16, 10>(m, r0, r1, w0, win_cap, m.resid + b, sh, invQ, bnd, obs); break;
-        default: drop_rows<32, 6>(m, r0, r1, w0, win_cap, m.resid + b, sh, invQ, bnd, obs); break;
+        case 8: drop_rows<8, 16>(m, r0, r1, w0, win_cap, m.resid + b, sh, ws.invQ, ws.bound); break;
+        case 16: drop_rows<16, 10>(m, r0, r1, w0, win_cap, m.resid + b, sh, ws.invQ, ws.bound); break;
+        default: drop_rows<32, 6>(m, r0, r1, w0, win_cap, m.resid + b, sh, ws.invQ, ws.bound); break;
     }
     if (w0 >= 0) {
         __syncthreads();
@@ -420,7 +404,7 @@ __device__ void drop_item(const MemberDev& m, int b, int idx, int win_cap, doubl
         for (int j = threadIdx.x; j < n; j += blockDim.x) {   // the window is zero again afterwards
             const int v = wint[j];
             if (v != 0) {
-                atomicAdd(m.delta + w0 + j, (float)v * Q);
+                atomicAdd(m.delta + w0 + j, (float)v * ws.Q);
                 wint[j] = 0;
             }
         }
@@ -520,11 +504,9 @@ __device__ void finish_phase(const CycleArgs& a, int r, int phase, int items, un
             ph = PH_GRAD;
             n += 1;
             break;
-        case PH_DROP:   // the block's next window bound: twice the largest |r / lambda| of this sweep
-            if (m.wstat) {
-                const float o = __uint_as_float(atomicExch(reinterpret_cast<unsigned*>(m.wstat + 2 * m.B + b), 0u));
-                if (o > 0.f) m.wstat[m.B + b] = 2.f * o;
-            }
+        case PH_DROP:   // the next block's window scale
+            *(volatile float*)m.rms =
+                (float)sqrt(*(volatile double*)(m.resid + b) / (double)(m.block_ptr[b + 1] - m.block_ptr[b]));
             ph = PH_DAPPLY;
             break;
         case PH_DAPPLY:
@@ -773,7 +755,7 @@ __global__ void count_kernel(const int64_t* __restrict__ rp, const int32_t* __re
 // bits so that an unsigned atomic max orders them: colsum[j] += |a_ij| and *amax = max |a_ij|
 __global__ void colsum_kernel(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                               const float* __restrict__ val, int64_t r0, int64_t r1, float* __restrict__ colsum,
-                              unsigned* __restrict__ amax) {
+                              WinStat* st) {
     const int64_t q0 = rp[r0], q1 = rp[r1];
     unsigned mx = 0u;
     for (int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < q1; q += (int64_t)gridDim.x * blockDim.x) {
@@ -782,7 +764,7 @@ __global__ void colsum_kernel(const int64_t* __restrict__ rp, const int32_t* __r
         mx = max(mx, __float_as_uint(a));
     }
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0 && mx) atomicMax(amax, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(reinterpret_cast<unsigned*>(&st->amax), mx);
 }
 
 // *out = max(*out, largest of v[0..n)) for non-negative v
@@ -794,15 +776,23 @@ __global__ void max_bits_kernel(const float* __restrict__ v, int64_t n, unsigned
     if ((threadIdx.x & 31) == 0 && mx) atomicMax(out, mx);
 }
 
-// *out = max over rows [r0, r1) of |b_i| / ||a_i||^2: the residual bound at x = 0, the first
-// sweep's window bound
-__global__ void seed_bound_kernel(const float* __restrict__ b, const float* __restrict__ inn, int64_t r0, int64_t r1,
-                                  unsigned* __restrict__ out) {
-    unsigned mx = 0u;
-    for (int64_t i = r0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < r1; i += (int64_t)gridDim.x * blockDim.x)
-        mx = max(mx, __float_as_uint(fabsf(b[i]) * inn[i]));
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0 && mx) atomicMax(out, mx);
+// the sums of ||a_i||^2 and |b_i| over rows [r0, r1), each over the number of rows as WinStat has them;
+// one CTA
+__global__ void __launch_bounds__(1024) row_stat_kernel(const float* __restrict__ b, const float* __restrict__ inn,
+                                                        int64_t r0, int64_t r1, WinStat* st) {
+    __shared__ double sh[32];
+    double a2 = 0.0, bs = 0.0;
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+        if (inn[i] > 0.f) a2 += 1.0 / (double)inn[i];
+        bs += (double)fabsf(b[i]);
+    }
+    a2 = block_sum(a2, sh);
+    bs = block_sum(bs, sh);
+    if (threadIdx.x == 0) {
+        const double rows = (double)(r1 - r0);
+        st->inv_norm2 = a2 > 0.0 ? (float)(rows / a2) : 0.f;
+        st->mean_b = (float)(bs / rows);
+    }
 }
 
 __global__ void inv_count_kernel(const int32_t* __restrict__ cnt, float* __restrict__ inv_s, int64_t n) {
@@ -1054,8 +1044,10 @@ int member_prep(ntvs_batch* bt, ntvs_batch::Member& mm, const void* x0, int x0_d
     if (M > 0) norm_kernel<<<grid_of(M * 32), 256, 0, s>>>(d.row_ptr, d.val, M, (float*)d.inv_norm2);
     int32_t* cnt = nullptr;
     BTRY(balloc(&cnt, sizeof(int32_t) * VI, "hit counts"));
-    BTRY(member_alloc(mm, (void**)&d.wstat, sizeof(float) * 4 * (size_t)B, "window statistics"));
-    cudaMemsetAsync(d.wstat, 0, sizeof(float) * 4 * (size_t)B, s);
+    BTRY(member_alloc(mm, (void**)&d.wstat, sizeof(WinStat) * (size_t)B + sizeof(float), "window statistics"));
+    cudaMemsetAsync(d.wstat, 0, sizeof(WinStat) * (size_t)B, s);
+    d.rms = reinterpret_cast<float*>(d.wstat + B);
+    cudaMemsetAsync(d.rms, 0xff, sizeof(float), s);   // NaN: no residuals seen yet
     for (int t = 0; t < B; ++t) {
         cudaMemsetAsync(cnt, 0, sizeof(int32_t) * VI, s);
         if (mm.block_ptr[t + 1] > mm.block_ptr[t]) {
@@ -1063,12 +1055,11 @@ int member_prep(ntvs_batch* bt, ntvs_batch::Member& mm, const void* x0, int x0_d
             // the window statistics: column sums of |a| into the (reused) count buffer as floats
             inv_count_kernel<<<grid_of(VI), 256, 0, s>>>(cnt, (float*)d.inv_s + (size_t)t * VI, VI);
             cudaMemsetAsync(cnt, 0, sizeof(int32_t) * VI, s);
-            unsigned* w = reinterpret_cast<unsigned*>(d.wstat);
             colsum_kernel<<<grid_of(nnz), 256, 0, s>>>(d.row_ptr, d.col, d.val, mm.block_ptr[t], mm.block_ptr[t + 1],
-                                                       reinterpret_cast<float*>(cnt), w + 3 * B + t);
-            max_bits_kernel<<<grid_of(VI), 256, 0, s>>>(reinterpret_cast<const float*>(cnt), VI, w + t);
-            seed_bound_kernel<<<grid_of(mm.block_ptr[t + 1] - mm.block_ptr[t]), 256, 0, s>>>(
-                d.b, d.inv_norm2, mm.block_ptr[t], mm.block_ptr[t + 1], w + B + t);
+                                                       reinterpret_cast<float*>(cnt), d.wstat + t);
+            max_bits_kernel<<<grid_of(VI), 256, 0, s>>>(reinterpret_cast<const float*>(cnt), VI,
+                                                          reinterpret_cast<unsigned*>(&d.wstat[t].lmax));
+            row_stat_kernel<<<1, 1024, 0, s>>>(d.b, d.inv_norm2, mm.block_ptr[t], mm.block_ptr[t + 1], d.wstat + t);
         } else {
             inv_count_kernel<<<grid_of(VI), 256, 0, s>>>(cnt, (float*)d.inv_s + (size_t)t * VI, VI);
         }
@@ -1590,6 +1581,7 @@ int ntvs_batch_finalize(ntvs_batch* bt, int max_cycles) {
                 BCUDA(cudaMemcpyAsync(d.x32, saved[i++], sizeof(float) * d.vm.vint, cudaMemcpyDeviceToDevice, s));
                 BCUDA(cudaMemcpyAsync(d.xh, saved[i++], sizeof(float) * d.V, cudaMemcpyDeviceToDevice, s));
                 BCUDA(cudaMemcpyAsync(d.xl, saved[i++], sizeof(float) * d.V, cudaMemcpyDeviceToDevice, s));
+                BCUDA(cudaMemsetAsync(d.rms, 0xff, sizeof(float), s));
             }
             BCUDA(cudaMemsetAsync(bt->dst, 0, sizeof(MemberState) * R, s));
             BCUDA(cudaMemsetAsync(bt->drun, 0, sizeof(RunState), s));

@@ -93,6 +93,33 @@ __device__ __forceinline__ void store_copies(const ImgCopies& c, int64_t j, doub
     store_copies(c, j, c.x32 ? (uint32_t)vox_internal(c.m, j) : 0u, v);
 }
 
+// Scale of an FP32 scatter window that accumulates in int32 (kept in shared memory, uniform over
+// the CTA, so that the row loop's registers hold the matrix entries): quantum Q = 1 / invQ; rows
+// with |r_i / lambda| above `bound` scatter globally (invQ = 0 sends every row there), which
+// keeps every window slot below 2^30 Q and every converted term below 2^22 in magnitude.
+struct WinScale {
+    float invQ, bound, Q;
+};
+
+// The scale for a block whose rows have the statistics st (WinStat), rms being the root mean
+// square residual of the block swept before it (NaN: none, the image was set since).  The bound
+// is 10 rms on a row of mean ||a||^2, never below 1/16 and never above 4 of the block's mean |b|,
+// and 1/4 of it without an rms: so the quantum follows the residuals of the image being swept,
+// is at most 4 mean |b| coarse whatever an earlier sweep saw, and rows of very short chords, whose
+// |r / lambda| is far above the others', scatter globally instead of coarsening them.
+// At 10 rms the error of a sweep against 64 bits is that of FP32 reductions (2.773e-8 of the image
+// at 200x200x16, 2M rows in detected order, both ways); at 4 mean |b| it would be 2.9e-8.
+// A scale taken inside the launch, from its own first rows, was exact about the image but cost 6
+// of 62 us a block of 100k rows (the other warps wait for it, or scatter globally until it stands).
+__device__ __forceinline__ WinScale win_scale(float lambda, const WinStat& st, float rms) {
+    float bound = rms >= 0.f ? 10.f * rms : 0.25f * st.mean_b;
+    if (st.mean_b > 0.f) bound = fminf(fmaxf(bound, 0.0625f * st.mean_b), 4.f * st.mean_b);
+    bound *= st.inv_norm2;
+    const float lam = fabsf(lambda), Q = lam * bound * st.lmax * 0x1p-30f, iq = 1.f / Q;
+    if (!(st.amax > 0.f && Q > 0.f && isfinite(Q) && isfinite(iq))) return WinScale{0.f, 0.f, 0.f};
+    return WinScale{iq, fminf(bound, 0x1p22f * Q / (lam * st.amax)), Q};
+}
+
 // %globaltimer in nanoseconds (the clock of every bounded device-side wait)
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;

@@ -23,13 +23,9 @@ namespace ntvs {
 
 template <typename T, int U>
 __global__ void __launch_bounds__(256) drop_apply_kernel(double* __restrict__ x, ImgCopies c, T* __restrict__ delta,
-                                                         const T* __restrict__ inv_s, int64_t V, float* wbound,
-                                                         float* wobs) {
-    if (wbound && blockIdx.x == 0 && threadIdx.x == 0) {   // the window bound of the next sweep
-        const float o = *wobs;
-        if (o > 0.f) *wbound = 2.f * o;
-        *wobs = 0.f;
-    }
+                                                         const T* __restrict__ inv_s, int64_t V,
+                                                         const double* resid_ss, double rows, float* rms) {
+    if (rms && blockIdx.x == 0 && threadIdx.x == 0) *rms = (float)sqrt(*resid_ss / rows);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j0 < V; j0 += U * stride) {
         double xv[U];
@@ -78,14 +74,14 @@ cudaError_t k_drop_block(const DropArgs& a, cudaStream_t s) {
 }
 
 cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const void* inv_s, int64_t V, int grid,
-                         float* wbound, float* wobs, cudaStream_t s) {
+                         const double* resid_ss, int64_t rows, float* rms, cudaStream_t s) {
     const bool many = vox_unrolled(V, grid);
     if (cdt == F64)
         (many ? drop_apply_kernel<double, kVoxUnroll> : drop_apply_kernel<double, 1>)<<<grid, 256, 0, s>>>(
-            x, c, (double*)delta, (const double*)inv_s, V, wbound, wobs);
+            x, c, (double*)delta, (const double*)inv_s, V, resid_ss, (double)rows, rms);
     else
         (many ? drop_apply_kernel<float, kVoxUnroll> : drop_apply_kernel<float, 1>)<<<grid, 256, 0, s>>>(
-            x, c, (float*)delta, (const float*)inv_s, V, wbound, wobs);
+            x, c, (float*)delta, (const float*)inv_s, V, resid_ss, (double)rows, rms);
     return cudaGetLastError();
 }
 

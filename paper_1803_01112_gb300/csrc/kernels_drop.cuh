@@ -119,17 +119,6 @@ struct Window {
     int W;
 };
 
-// Scale of the FP32 fixed-point window, uniform over the CTA (kept in shared memory so
-// that the row loop's registers hold the matrix entries): quantum Q = 1 / invQ; rows with
-// |r_i / lambda| above `bound` scatter globally (invQ = 0 sends every row there), which
-// keeps every window slot below 2^30 Q and every converted term below 2^22 in magnitude;
-// `obs` collects the largest |r_i / lambda| seen (float bits, atomic max).
-struct WinScale {
-    float invQ;
-    float bound;
-    unsigned obs;
-};
-
 // A DELTA16 word read without allocating in L1, which the x gathers then keep (0.2504 ->
 // 0.2481 ms per 500k-row BF16 block; the FP32 pairs measured slower this way, 0.2307 ->
 // 0.2325 ms, and keep the streaming load)
@@ -157,22 +146,17 @@ __device__ __forceinline__ void scatter(T* delta, const Window& w, int32_t c, T 
 }
 
 // the row's r = lambda * res / ||a||^2, whether its windowed entries go to the fixed-point
-// window, and r / Q; the row's first lane records |res / ||a||^2| of a valid row in ws->obs
+// window, and r / Q
 template <typename T, bool WIN>
-__device__ __forceinline__ void row_factor(bool valid, bool first_lane, T res, T inv, T lambda, WinScale* ws,
-                                           T& r, bool& rowfix, float& rq) {
+__device__ __forceinline__ void row_factor(T res, T inv, T lambda, const WinScale* ws, T& r, bool& rowfix, float& rq) {
     const T rn = res * inv;
     r = lambda * rn;
     rowfix = false;
     rq = 0.f;
     if constexpr (WIN) {
-        const float arn = fabsf((float)rn);
         const float iq = ws->invQ;
-        rowfix = iq > 0.f && arn <= ws->bound;
+        rowfix = iq > 0.f && fabsf((float)rn) <= ws->bound;
         rq = (float)r * iq;
-        // the block's largest |r/lambda|: a plain read first skips the atomic for most rows
-        if (valid && first_lane && __float_as_uint(arn) > *(volatile unsigned*)&ws->obs)
-            atomicMax(&ws->obs, __float_as_uint(arn));
     }
 }
 
@@ -321,7 +305,7 @@ __device__ __forceinline__ void drop_row(int64_t i, const RowHead& h, bool valid
     T r;
     bool rowfix;
     float rq;
-    row_factor<T, WIN>(valid, sub == 0, res, inv, lambda, ws, r, rowfix, rq);
+    row_factor<T, WIN>(res, inv, lambda, ws, r, rowfix, rq);
 #pragma unroll
     for (int u = 0; u < CH; ++u)
 #pragma unroll
@@ -452,8 +436,8 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
                          const V* __restrict__ val, const T* __restrict__ b, const T* __restrict__ inv_norm2,
                          const DropSegment* __restrict__ segs, const int32_t* __restrict__ seg_begin,
                          int64_t slice, const T* __restrict__ x, T* __restrict__ delta, T lambda,
-                         double* resid_ss, Delta16 d16, const float* wlmax, const float* wbound, float* wobs,
-                         const float* wamax, const int32_t* __restrict__ row_order) {
+                         double* resid_ss, Delta16 d16, const WinStat* wstat, const float* wrms,
+                         const int32_t* __restrict__ row_order) {
     static_assert(!ORD || (!D16 && sizeof(T) == 4 && 20 * kOrderedStage <= stage_bytes_all<float, false>()),
                   "ordered rows are packed FP32 pairs and stage in the space of the others");
     constexpr int RS = ORD ? kOrderedStage : row_stage<D16>();
@@ -467,18 +451,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
     const int nwarps = blockDim.x >> 5;
     for (int j = threadIdx.x; j < W; j += blockDim.x) win[j] = 0;
     for (int q = threadIdx.x; q < 32 * G; q += blockDim.x) (&ss_grp[0][0])[q] = 0.0;
-    // rows with |r/lambda| <= bound keep |window slot| <= |lambda| bound lmax = 2^30 Q (no
-    // int32 overflow); rows also below 2^22 Q / (|lambda| amax) keep every term below 2^22
-    const float bound = wbound ? *wbound : 0.f, lmax = wlmax ? *wlmax : 0.f, amax = wamax ? *wamax : 0.f;
-    const float lam = fabsf((float)lambda);
-    const float Q = lam * bound * lmax * 0x1p-30f;
-    if (threadIdx.x == 0) {
-        const float iq = 1.f / Q;
-        const bool fix = bound > 0.f && amax > 0.f && Q > 0.f && isfinite(Q) && isfinite(iq);
-        ws.invQ = fix ? iq : 0.f;
-        ws.bound = fix ? fminf(bound, 0x1p22f * Q / (lam * amax)) : 0.f;
-        ws.obs = 0u;
-    }
+    if (threadIdx.x == 0) ws = win_scale((float)lambda, *wstat, *wrms);
     __syncthreads();
     const int s0 = seg_begin[blockIdx.x], s1 = seg_begin[blockIdx.x + 1];
     int cur = s0 < s1 ? segs[s0].home : 0;
@@ -488,7 +461,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
         const DropSegment sg = segs[s];
         if (sg.home != cur) {   // uniform across the CTA
             __syncthreads();
-            flush_window(win, W, delta, w.w0, Q);
+            flush_window(win, W, delta, w.w0, ws.Q);
             __syncthreads();
             cur = sg.home;
             w.w0 = (int)(cur * slice);
@@ -558,14 +531,11 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
         }
     }
     __syncthreads();
-    flush_window(win, W, delta, w.w0, Q);
+    flush_window(win, W, delta, w.w0, ws.Q);
     if (lane < G) ss = ss_grp[warp][lane];
     __shared__ double sh[32];
     const double tot = block_sum(ss, sh);   // synchronizes the CTA
-    if (threadIdx.x == 0) {
-        if (tot != 0.0) atomicAdd(resid_ss, tot);
-        if (wobs && ws.obs) atomicMax(reinterpret_cast<unsigned*>(wobs), ws.obs);
-    }
+    if (threadIdx.x == 0 && tot != 0.0) atomicAdd(resid_ss, tot);
 }
 
 // ------------------------------------------------------------------ launch
@@ -577,7 +547,7 @@ cudaError_t launch_window(const DropArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     kern<<<a.grid, 1024, smem, s>>>(a.row_ptr, a.col, (const V*)a.val, (const T*)a.b, (const T*)a.inv_norm2, a.segs,
                                     a.seg_begin, a.slice, (const T*)a.x, (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16,
-                                    a.wlmax, a.wbound, a.wobs, a.wamax, a.order);
+                                    a.wstat, a.wrms, a.order);
     return cudaGetLastError();
 }
 

@@ -75,9 +75,8 @@ namespace ntvs {
 // row), and the hit counts of the entries with a != 0.  Requires a validated row_ptr.
 // FP64 path (cs null): cnt[j] += 1.
 // FP32 path (cs not null): cs[j] += {1, |a_ij|}, the hit count and the block's column sum of
-// lengths with one two-element reduction; rb[0] = max
-// over the rows of |b_i| / ||a_i||^2 and rb[1] = max |a_ij| (as float bits, atomic maxima of
-// non-negative floats): the scale statistics of the fixed-point DROP window.  A count is
+// lengths with one two-element reduction; st takes the largest |a_ij| (an atomic maximum of the
+// bits of non-negative floats) and the sums of ||a_i||^2 and |b_i|.  A count is
 // exact below 2^24, where it stays; finish_block_kernel reports it.
 // PACK (FP32 values in CSR32 storage): col holds canonical columns; entry p leaves as the pair
 // {internal column, value bits} in ent[p], so columns and values are read once and never
@@ -89,13 +88,13 @@ __global__ void __launch_bounds__(256) prep_block_kernel(const int64_t* __restri
                                                          int64_t e0, const T* __restrict__ b, int64_t r0, int64_t r1,
                                                          int64_t nvox, VoxMap vm, T* __restrict__ inv_norm2,
                                                          int32_t* __restrict__ cnt, int* flags,
-                                                         float2* __restrict__ cs, unsigned* rb,
+                                                         float2* __restrict__ cs, WinStat* st,
                                                          int2* __restrict__ ent) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     int f = 0;
-    float bmax = 0.f, amax = 0.f;
+    float amax = 0.f, asum = 0.f, bsum = 0.f;
     for (int64_t i = r0 + w0; i < r1; i += nw) {
         const int64_t p0 = __ldg(row_ptr + i), p1 = __ldg(row_ptr + i + 1);
         double sq = 0.0;
@@ -128,25 +127,28 @@ __global__ void __launch_bounds__(256) prep_block_kernel(const int64_t* __restri
             inv_norm2[i] = (T)inv;
             const double bi = (double)b[i];
             if (!isfinite(bi)) f |= 16;
-            else bmax = fmaxf(bmax, (float)(fabs(bi) * inv));
+            asum += (float)sq;
+            bsum += (float)fabs(bi);
         }
     }
     if (f) atomicOr(flags, f);
-    if (rb) {
-        for (int o = 16; o > 0; o >>= 1) {
-            bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
-            amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        }
-        if (lane == 0 && bmax > 0.f) atomicMax(rb, __float_as_uint(bmax));
-        if (lane == 0 && amax > 0.f) atomicMax(rb + 1, __float_as_uint(amax));
+    if (st) {
+        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        if (lane == 0 && amax > 0.f) atomicMax(reinterpret_cast<unsigned*>(&st->amax), __float_as_uint(amax));
+        if (lane == 0 && asum > 0.f) atomicAdd(&st->inv_norm2, asum);
+        if (lane == 0 && bsum > 0.f) atomicAdd(&st->mean_b, bsum);
     }
 }
 
 // A block's counts and column sums once its rows are through: inv_s[j] = 1 / count (0 for an
-// unhit voxel), *lmax = max_j of the sums, and cs cleared for the next block; flags |= 64 when
-// a count reached 2^24.
+// unhit voxel), st->lmax = max_j of the sums, and cs cleared for the next block; the row sums in st
+// become means; flags |= 64 when a count reached 2^24.
 __global__ void __launch_bounds__(256) finish_block_kernel(float2* __restrict__ cs, int64_t n, float* __restrict__ inv_s,
-                                                           unsigned* lmax, int* flags) {
+                                                           WinStat* st, float rows, int* flags) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->inv_norm2 = st->inv_norm2 > 0.f ? rows / st->inv_norm2 : 0.f;
+        st->mean_b /= rows;
+    }
     float m = 0.f;
     bool full = false;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
@@ -157,15 +159,16 @@ __global__ void __launch_bounds__(256) finish_block_kernel(float2* __restrict__ 
         m = fmaxf(m, v.y);
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(lmax, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned*>(&st->lmax), __float_as_uint(m));
     if (full) atomicOr(flags, 64);
 }
 
-cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, float* lmax, int* flags, cudaStream_t s) {
+cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, WinStat* st, int64_t rows, int* flags,
+                           cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int64_t need = (n + 255) / 256;
     const int grid = (int)(need < prep_grid() ? need : prep_grid());
-    finish_block_kernel<<<grid, 256, 0, s>>>(cs, n, inv_s, reinterpret_cast<unsigned*>(lmax), flags);
+    finish_block_kernel<<<grid, 256, 0, s>>>(cs, n, inv_s, st, (float)(rows > 0 ? rows : 1), flags);
     return cudaGetLastError();
 }
 
@@ -190,18 +193,17 @@ cudaError_t k_recount(const int64_t* row_ptr, int64_t r0, int64_t r1, const int3
 template <typename V, typename T, bool PACK>
 static cudaError_t launch_prep(const int64_t* rp, const int32_t* col, const void* val, int64_t e0, const void* b,
                                int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inn, int32_t* cnt,
-                               int* flags, float2* cs, float* rb, int32_t* ent, cudaStream_t s) {
+                               int* flags, float2* cs, WinStat* st, int32_t* ent, cudaStream_t s) {
     prep_block_kernel<V, T, PACK><<<prep_grid(), 256, 0, s>>>(rp, col, (const V*)val, e0, (const T*)b, r0, r1, nvox, vm,
-                                                             (T*)inn, cnt, flags, cs, reinterpret_cast<unsigned*>(rb),
-                                                             reinterpret_cast<int2*>(ent));
+                                                             (T*)inn, cnt, flags, cs, st, reinterpret_cast<int2*>(ent));
     return cudaGetLastError();
 }
 
 cudaError_t k_prep_block(const int64_t* row_ptr, const int32_t* col, const void* val, int64_t e0, int vdt,
                          const void* b, int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inv_norm2,
-                         int cdt, int32_t* cnt, int* flags, float2* cs, float* rb, int32_t* ent, cudaStream_t s) {
+                         int cdt, int32_t* cnt, int* flags, float2* cs, WinStat* st, int32_t* ent, cudaStream_t s) {
     if (r1 <= r0) return cudaSuccess;
-#define NTVS_PREP(V, T, P) launch_prep<V, T, P>(row_ptr, col, val, e0, b, r0, r1, nvox, vm, inv_norm2, cnt, flags, cs, rb, ent, s)
+#define NTVS_PREP(V, T, P) launch_prep<V, T, P>(row_ptr, col, val, e0, b, r0, r1, nvox, vm, inv_norm2, cnt, flags, cs, st, ent, s)
     if (cdt == F64) {
         if (vdt == F64) return NTVS_PREP(double, double, false);
         if (vdt == F32) return ent ? NTVS_PREP(float, double, true) : NTVS_PREP(float, double, false);

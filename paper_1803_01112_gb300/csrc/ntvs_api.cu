@@ -115,8 +115,8 @@ struct ntvs_ctx {
     DropStage* stages = nullptr;       // pipelined schedule: all blocks' stages
     int32_t* stage_begin = nullptr;    // [B][win_grid + 1]
     int win_grid = 0;
-    float* wstat = nullptr;            // FP32 window scale per block: lmax [B], bound [B], observed [B],
-                                       // then per block the seed bound and max |a| [2B]
+    WinStat* wstat = nullptr;          // FP32: [B] statistics of the blocks' rows (scale of the window)
+    float* wrms = nullptr;             // FP32: rms residual of the last swept block (NaN: none since set_image)
     int* derr = nullptr;               // device error word (bounded waits that ran out)
     // DELTA16 index storage (packed at load from the int32 columns)
     uint16_t* d16off = nullptr;        // [nnz] column - chunk base
@@ -218,6 +218,7 @@ struct ntvs_ctx {
         dev_free(seg_begin);
         dev_free(order);
         dev_free(wstat);
+        dev_free(wrms);
         dev_free(stages);
         dev_free(stage_begin);
         dev_free(d16off);
@@ -529,10 +530,8 @@ int perturb_steps(ntvs_ctx* c, int64_t* ell_io) {
 // Launches the DROP gather + scatter kernel of rows [r0, r1) of block t into delta
 // (nothing applied), its residual sum of squares into *resid.  The whole block runs the
 // context's schedule; a proper sub-range of it runs the plain schedule (the windowed and
-// pipelined plans cover whole blocks).  *wb / *wo receive the block's window-scale slots
-// for the apply kernel (null when the schedule has none).
-int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid, float** wb, float** wo) {
-    *wb = *wo = nullptr;
+// pipelined plans cover whole blocks).
+int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid) {
     if (r1 <= r0) return NTVS_OK;
     const bool whole = r0 == c->block_ptr[t] && r1 == c->block_ptr[t + 1];
     if (c->paths_mode) {
@@ -565,22 +564,14 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
     a.seg_begin = nullptr;
     a.order = nullptr;
     a.slice = c->vm.slice_p;
-    a.wlmax = nullptr;
-    a.wbound = nullptr;
-    a.wobs = nullptr;
-    a.wamax = nullptr;
+    a.wstat = c->wstat ? c->wstat + t : nullptr;
+    a.wrms = c->wrms;
     a.max_row = t < (int)c->block_maxrow.size() ? c->block_maxrow[t] : (int64_t)1 << 40;
     if (whole && c->schedule == NTVS_SCHED_WINDOW && c->segs) {
         a.segs = c->segs;
         a.order = c->order;
         a.seg_begin = c->seg_begin + (size_t)t * (c->win_grid + 1);
         a.grid = c->win_grid;
-        if (c->wstat) {
-            a.wlmax = c->wstat + t;
-            a.wbound = *wb = c->wstat + c->B + t;
-            a.wobs = *wo = c->wstat + 2 * c->B + t;
-            a.wamax = c->wstat + 3 * c->B + 2 * t + 1;
-        }
     }
     if (whole && c->schedule == NTVS_SCHED_PIPELINE) {
         DropPipeArgs pa;
@@ -621,9 +612,7 @@ int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
     const bool split = t == c->B - 1;
     if (!resid_cleared) CUDA_TRY(cudaMemsetAsync(c->resid + t, 0, sizeof(double), c->stream));
     if (r1 <= r0 && !c->ar_fn) return NTVS_OK;
-    float* wb = nullptr;
-    float* wo = nullptr;
-    TRY(launch_drop_kernel(c, t, r0, r1, c->resid + t, &wb, &wo));
+    TRY(launch_drop_kernel(c, t, r0, r1, c->resid + t));
     if (c->ar_fn) {
         int rc = c->ar_fn(c->delta, c->vm.vint, c->cdt, (void*)c->stream, c->ar_user);
         if (rc == 0) rc = c->ar_fn(c->resid + t, 1, NTVS_F64, (void*)c->stream, c->ar_user);
@@ -633,8 +622,8 @@ int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
     }
     CUDA_TRY(timed_launch(c, KIND_APPLY, [&] {
         return k_drop_apply(c->cdt, c->x, c->copies(split), c->delta,
-                            (const char*)c->inv_s + (size_t)t * c->vm.vint * c->csz(), c->V, c->apply_grid, wb, wo,
-                            c->stream);
+                            (const char*)c->inv_s + (size_t)t * c->vm.vint * c->csz(), c->V, c->apply_grid,
+                            c->resid + t, r1 - r0, r1 > r0 ? c->wrms : nullptr, c->stream);
     }));
     c->split_stale = !split;
     return NTVS_OK;
@@ -1282,8 +1271,7 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     TRY(dev_alloc(&c->inv_norm2, csz * (size_t)M, "inv_norm2"));
     // hit counts: integers for all blocks at once (FP64), or (FP32) one block's counts beside its
     // column sums of |a_ij|, from which come the inverse counts and the scale statistics of the
-    // fixed-point DROP window (lmax = the largest column sum, the bound seeded with
-    // max_i |b_i| / ||a_i||^2)
+    // fixed-point DROP window
     int32_t* cnt = nullptr;
     float2* cs = nullptr;
     struct FreeCounts {
@@ -1293,8 +1281,10 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     } counts_guard{cnt, cs};
     TRY(dev_alloc(&c->inv_s, csz * (size_t)c->B * VI, "inverse hit counts"));
     if (c->cdt == F32) {
-        TRY(dev_alloc(&c->wstat, sizeof(float) * 5 * (size_t)c->B, "window scale statistics"));
-        CUDA_TRY(cudaMemsetAsync(c->wstat, 0, sizeof(float) * 5 * (size_t)c->B, st));
+        TRY(dev_alloc(&c->wstat, sizeof(WinStat) * (size_t)c->B, "window scale statistics"));
+        CUDA_TRY(cudaMemsetAsync(c->wstat, 0, sizeof(WinStat) * (size_t)c->B, st));
+        TRY(dev_alloc(&c->wrms, sizeof(float), "rms residual"));
+        CUDA_TRY(cudaMemsetAsync(c->wrms, 0x7f, sizeof(float), st));   // 3.4e38: at x = 0 the residual is b
         TRY(dev_alloc(&cs, sizeof(float2) * (size_t)VI, "hit counts and column sums"));
         CUDA_TRY(cudaMemsetAsync(cs, 0, sizeof(float2) * (size_t)VI, st));
     } else {
@@ -1318,8 +1308,10 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
         }
         CUDA_TRY(k_prep_block(c->row_ptr, bc, bv, e0, c->vdt, c->b, bp[t], bp[t + 1], pack ? V : VI, c->vm,
                               c->inv_norm2, c->cdt, cnt ? cnt + (size_t)t * VI : nullptr, c->dflags, cs,
-                              cs ? c->wstat + 3 * c->B + 2 * t : nullptr, c->ent, st));
-        if (cs) CUDA_TRY(k_finish_block(cs, VI, (float*)c->inv_s + (size_t)t * VI, c->wstat + t, c->dflags, st));
+                              cs ? c->wstat + t : nullptr, c->ent, st));
+        if (cs)
+            CUDA_TRY(k_finish_block(cs, VI, (float*)c->inv_s + (size_t)t * VI, c->wstat + t, bp[t + 1] - bp[t],
+                                    c->dflags, st));
         if (ring) {   // the slot is free again: the block nslots on may be copied into it
             cudaEvent_t ev;
             CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -1340,14 +1332,6 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
         dev_free(dm);
         if (e != cudaSuccess) return fail(NTVS_ERR_CUDA, cuda_msg("row lengths", e));
         c->block_maxrow.assign(hm.begin(), hm.end());
-    }
-    if (c->wstat) {   // the first sweep's bound: max |b_i| / ||a_i||^2 (the residual at x = 0)
-        std::vector<float> ws((size_t)5 * c->B);
-        CUDA_TRY(cudaMemcpyAsync(ws.data(), c->wstat, sizeof(float) * ws.size(), cudaMemcpyDeviceToHost, st));
-        CUDA_TRY(cudaStreamSynchronize(st));
-        for (int t = 0; t < c->B; ++t) ws[(size_t)c->B + t] = ws[(size_t)3 * c->B + 2 * t];
-        CUDA_TRY(cudaMemcpyAsync(c->wstat, ws.data(), sizeof(float) * ws.size(), cudaMemcpyHostToDevice, st));
-        CUDA_TRY(cudaStreamSynchronize(st));
     }
     CUDA_TRY(cudaMemcpyAsync(c->hint, c->dflags, sizeof(int), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -1641,6 +1625,7 @@ int ntvs_set_image(ntvs_ctx* c, const void* x, int dtype, int mem_kind) {
         CUDA_TRY(cudaStreamSynchronize(c->stream));
     }
     if (c->x32) CUDA_TRY(k_x32_from_x64(c->x, c->copies(), c->stream));
+    if (c->wrms) CUDA_TRY(cudaMemsetAsync(c->wrms, 0xff, sizeof(float), c->stream));   // NaN: no residuals seen yet
     c->split_stale = false;
     return NTVS_OK;
 }
@@ -1988,9 +1973,7 @@ int ntvs_drop_block_partial(ntvs_ctx* c, int t, int64_t r0, int64_t r1, void* de
     if (r0 < c->block_ptr[t] || r1 > c->block_ptr[t + 1] || r0 > r1)
         return fail(NTVS_ERR_ARG, "rows [r0, r1) must lie inside block t");
     CUDA_TRY(cudaMemsetAsync(c->dscal + 4, 0, sizeof(double), c->stream));
-    float* wb = nullptr;
-    float* wo = nullptr;
-    TRY(launch_drop_kernel(c, t, r0, r1, c->dscal + 4, &wb, &wo));
+    TRY(launch_drop_kernel(c, t, r0, r1, c->dscal + 4));
     const size_t bytes = (size_t)c->V * dt_size(dtype);
     if (mem_kind == NTVS_MEM_DEVICE) {
         CUDA_TRY(k_delta_out(c->cdt, c->delta, c->vm, delta_out, dtype, c->stream));

@@ -102,21 +102,30 @@ constexpr int kRedThreads = 256;
 int red_grid(int64_t n, int sm_count);
 
 // ------------------------------------------------------------------ load-time prep
+// A block's row statistics for the scale of the fixed-point scatter window (WinScale)
+struct WinStat {
+    float lmax;        // largest column sum of |a_ij|
+    float amax;        // largest |a_ij|
+    float inv_norm2;   // rows / sum of ||a_i||^2 (while the block is prepared: the sum)
+    float mean_b;      // mean |b_i| (while the block is prepared: the sum)
+};
+
 // flags |= 1 if row_ptr decreases, 2 if row_ptr[0] != 0
 cudaError_t k_validate_rows(const int64_t* row_ptr, int64_t M, int* flags, cudaStream_t s);
 // fused pass over the rows [r0, r1) of one block: validation of columns (against [0, nvox)),
 // values and b (flags 4 / 8 / 16), inv_norm2 of the rows and the block's hit counts: cnt[j] += 1,
-// or with cs (FP32 path) cs[j] += {1, |a_ij|}, rb[0] = max(rb[0], max_i |b_i| / ||a_i||^2) and
-// rb[1] = max(rb[1], max |a_ij|).  col and val hold the entries from e0 on: entry p is
+// or with cs (FP32 path) cs[j] += {1, |a_ij|} and *st takes the block's largest |a_ij| and the sums
+// of ||a_i||^2 and |b_i|.  col and val hold the entries from e0 on: entry p is
 // col[p - e0] (0 for whole arrays, the block's first entry for a staging slot).  With ent (FP32
 // values in CSR32 storage) col is canonical and entry p is also packed into pair p of ent, its
 // column in the order of vm; without it col is in that order already.
 cudaError_t k_prep_block(const int64_t* row_ptr, const int32_t* col, const void* val, int64_t e0, int vdt,
                          const void* b, int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inv_norm2,
-                         int cdt, int32_t* cnt, int* flags, float2* cs, float* rb, int32_t* ent, cudaStream_t s);
-// inv_s = 1 / hit count from cs, *lmax = max(*lmax, largest column sum), cs cleared;
-// flags |= 64 when a count reached 2^24 (recount then)
-cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, float* lmax, int* flags, cudaStream_t s);
+                         int cdt, int32_t* cnt, int* flags, float2* cs, WinStat* st, int32_t* ent, cudaStream_t s);
+// inv_s = 1 / hit count from cs, st->lmax = the largest column sum, st's sums over the block's rows
+// turned into means, cs cleared; flags |= 64 when a count reached 2^24 (recount then)
+cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, WinStat* st, int64_t rows, int* flags,
+                           cudaStream_t s);
 // cnt[j] += hits of the packed entries of rows [r0, r1)
 cudaError_t k_recount(const int64_t* row_ptr, int64_t r0, int64_t r1, const int32_t* ent, int32_t* cnt, cudaStream_t s);
 // col_out[p] = internal index of voxel col_in[p]; flags |= 4 for a column outside [0, V)
@@ -220,15 +229,10 @@ struct DropArgs {
     const int32_t* seg_begin;
     const int32_t* order;   // not null: segments are runs of positions in this row order
     int64_t slice;
-    // FP32 windowed schedule: the window accumulates in int32 fixed point with quantum
-    // Q = |lambda| * bound * lmax / 2^30, where lmax = max_j sum_{i in block} |a_ij| and
-    // bound = *wbound (a bound on |b_i - <a_i,x>| / ||a_i||^2); rows above the bound
-    // scatter with global FP32 reductions instead.  *wobs receives the block's observed
-    // max of that ratio (atomic max of float bits).  All three point at block t's slot.
-    const float* wlmax;
-    const float* wbound;
-    float* wobs;
-    const float* wamax;   // max |a_ij| of the block: rows whose terms could reach 2^22 Q go global
+    // FP32 windowed schedule: the window accumulates in int32 fixed point; its scale comes from the
+    // block's statistics and the rms residual of the block swept before (WinScale)
+    const WinStat* wstat;
+    const float* wrms;
     int64_t max_row;      // longest row of the block (register steps of the windowed kernel)
 };
 // dynamic shared memory of the windowed DROP kernel for a slice of `slice` voxels
@@ -280,10 +284,10 @@ cudaError_t k_row_home(const int64_t* row_ptr, const int32_t* col, int stride, i
 cudaError_t k_chunk_home(const int32_t* home, const int64_t* chunk_start, int64_t nchunks, int32_t* out,
                          unsigned long long* changes, int grid, cudaStream_t s);
 // x_j += delta_p * inv_s_p on the FP64 master (p the internal index of j) and its FP32
-// copies; delta_p = 0.  With wbound (block t's slot, nullable): *wbound = 2 * *wobs when
-// the block observed a ratio (the next sweep's bound), *wobs = 0.
+// copies; delta_p = 0.  With rms not null also *rms = sqrt(*resid_ss / rows), the block's root mean
+// square residual.
 cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const void* inv_s, int64_t V, int grid,
-                         float* wbound, float* wobs, cudaStream_t s);
+                         const double* resid_ss, int64_t rows, float* rms, cudaStream_t s);
 
 // TMA-fed pipeline (drop_pipe_kernel): a stage is a run of at most kStageRows whole rows
 // of one home slice whose entries [e0, e0 + nent) fit one ring slot (e0 and nent aligned
