@@ -941,8 +941,6 @@ struct ntvs_batch {
     double* part2 = nullptr;
     double* part_try = nullptr;
     double* beta = nullptr;          // [N_max][R]
-    float* stage = nullptr;          // FP32 image on its way to the host (the largest one asked for)
-    size_t stage_bytes = 0;
     double* hbeta[2] = {nullptr, nullptr};
     int N_max = 0;
     int total_vox_items = 0;
@@ -1282,7 +1280,6 @@ int ntvs_batch_destroy(ntvs_batch* bt) {
     cudaFree(bt->part2);
     cudaFree(bt->part_try);
     cudaFree(bt->beta);
-    cudaFree(bt->stage);
     for (int j = 0; j < 2; ++j) {
         if (bt->hbeta[j]) cudaFreeHost(bt->hbeta[j]);
         if (bt->graph[j]) cudaGraphExecDestroy(bt->graph[j]);
@@ -1714,24 +1711,19 @@ int ntvs_batch_get_image(ntvs_batch* bt, int index, void* out, int dtype, int me
     if (mem_kind != NTVS_MEM_HOST && mem_kind != NTVS_MEM_DEVICE) return bfail(NTVS_ERR_ARG, "bad mem_kind");
     BTRY(ntvs_batch_sync(bt));
     const MemberDev& d = bt->m[index].d;
-    // converted on the device, straight into a device output or through a buffer of the batch
+    // on the legacy stream, behind the caller's pending default-stream work on out (the batch's
+    // own stream does not wait for it); FP32 is converted into the member's gradient first, which
+    // every step forms anew
+    cudaStream_t st = cudaStreamLegacy;
     const size_t bytes = (dtype == NTVS_F64 ? sizeof(double) : sizeof(float)) * (size_t)d.V;
-    if (mem_kind == NTVS_MEM_DEVICE) {
-        BCUDA(k_convert(d.x, F64, out, dtype, d.V, bt->stream));
-    } else if (dtype == NTVS_F64) {
-        BCUDA(cudaMemcpyAsync(out, d.x, bytes, cudaMemcpyDeviceToHost, bt->stream));
-    } else {
-        if (bt->stage_bytes < bytes) {
-            cudaFree(bt->stage);
-            bt->stage = nullptr;
-            bt->stage_bytes = 0;
-            BTRY(balloc(&bt->stage, bytes, "image read-back"));
-            bt->stage_bytes = bytes;
-        }
-        BCUDA(k_convert(d.x, F64, bt->stage, F32, d.V, bt->stream));
-        BCUDA(cudaMemcpyAsync(out, bt->stage, bytes, cudaMemcpyDeviceToHost, bt->stream));
+    const void* src = d.x;
+    if (dtype == NTVS_F32) {
+        BCUDA(k_convert(d.x, F64, d.g, F32, d.V, st));
+        src = d.g;
     }
-    BCUDA(cudaStreamSynchronize(bt->stream));
+    BCUDA(cudaMemcpyAsync(out, src, bytes, mem_kind == NTVS_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                          st));
+    BCUDA(cudaStreamSynchronize(st));
     return NTVS_OK;
 }
 
