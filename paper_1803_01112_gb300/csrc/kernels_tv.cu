@@ -108,25 +108,38 @@ tv_grad_tile_kernel(const double* __restrict__ x, double* __restrict__ g, int nx
     }
 }
 
-// FP32 path: the gradient from the split copies xh + xl of the master image, one thread per
-// voxel: every neighbour difference is (xh_a - xh_b) + (xl_a - xl_b) in FP32, so the stencil
-// runs without FP64 arithmetic (only ||g||^2 is accumulated in FP64).  PHI: also phi_0(x) from the
-// master image, its three differences and square root being the pass's only FP64 stencil work
-// (with every difference of the gradient taken in FP64 too, 31.7 us on 128x128x16; 29.5 us).
+// FP32 path, one thread per voxel: neighbour differences as FP32 numbers, the rest of the stencil
+// in FP32, ||g||^2 accumulated in FP64.  Without PHI every difference is (xh_a - xh_b) +
+// (xl_a - xl_b) from the split copies of the master image, so the stencil runs without FP64
+// arithmetic.  PHI: also phi_0(x), whose differences are formed in FP64 from the master image; the
+// gradient's are those, rounded once (128x128x16: 31.8 us so and 28.6 with the split ones, which
+// lose what xl has no bits for, 2^-49 of the voxel).
 template <bool PHI>
 __global__ void __launch_bounds__(kRedThreads)
-tv_grad_split_kernel(const double* __restrict__ x, const float* __restrict__ xh, const float* __restrict__ xl, float* __restrict__ g, int nx,
-                     int ny, int nz, float eps, double* partials, unsigned* ticket, double* gnorm2, double* phi) {
+tv_grad_f32_kernel(const double* __restrict__ x, const float* __restrict__ xh, const float* __restrict__ xl,
+                   float* __restrict__ g, int nx, int ny, int nz, float eps, double* partials, unsigned* ticket,
+                   double* gnorm2, double* phi) {
     const int64_t sxy = (int64_t)nx * ny, V = sxy * nz;
     auto dif = [&](int64_t a, int64_t b) -> float {
-        return (__ldg(xh + a) - __ldg(xh + b)) + (__ldg(xl + a) - __ldg(xl + b));
+        if constexpr (PHI) return (float)(__ldg(x + a) - __ldg(x + b));
+        else return (__ldg(xh + a) - __ldg(xh + b)) + (__ldg(xl + a) - __ldg(xl + b));
     };
     double acc[PHI ? 2 : 1] = {};
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < V; p += (int64_t)gridDim.x * blockDim.x) {
         int ix, iy, iz;
         voxel_coords(p, nx, ny, ix, iy, iz);
         const bool hx = ix + 1 < nx, hy = iy + 1 < ny, hz = iz + 1 < nz;
-        const float dx = hx ? dif(p + 1, p) : 0.f, dy = hy ? dif(p + nx, p) : 0.f, dz = hz ? dif(p + sxy, p) : 0.f;
+        double ex = 0.0, ey = 0.0, ez = 0.0;
+        float dx, dy, dz;
+        if constexpr (PHI) {
+            const double xc = __ldg(x + p);
+            ex = hx ? __ldg(x + p + 1) - xc : 0.0;
+            ey = hy ? __ldg(x + p + nx) - xc : 0.0;
+            ez = hz ? __ldg(x + p + sxy) - xc : 0.0;
+            dx = (float)ex, dy = (float)ey, dz = (float)ez;
+        } else {
+            dx = hx ? dif(p + 1, p) : 0.f, dy = hy ? dif(p + nx, p) : 0.f, dz = hz ? dif(p + sxy, p) : 0.f;
+        }
         const float D = sqrtf(eps + (dx * dx + dy * dy + dz * dz));
         float gq = (D > 0.f) ? -(dx + dy + dz) / D : 0.f;
         if (ix > 0) {
@@ -149,12 +162,7 @@ tv_grad_split_kernel(const double* __restrict__ x, const float* __restrict__ xh,
         }
         g[p] = gq;
         acc[0] += (double)gq * (double)gq;
-        if constexpr (PHI) {
-            const double xc = __ldg(x + p);
-            const double ex = hx ? __ldg(x + p + 1) - xc : 0.0, ey = hy ? __ldg(x + p + nx) - xc : 0.0,
-                         ez = hz ? __ldg(x + p + sxy) - xc : 0.0;
-            acc[1] += sqrt(ex * ex + ey * ey + ez * ez);
-        }
+        if constexpr (PHI) acc[1] += sqrt(ex * ex + ey * ey + ez * ez);
     }
     if constexpr (PHI) {
         double* const outs[2] = {gnorm2, phi};
@@ -293,8 +301,8 @@ cudaError_t k_tv_grad(int cdt, const double* x, const float* xh, const float* xl
                              : (phi ? launch_grad_tile<true, 16> : launch_grad_tile<false, 16>);
         return run(x, (double*)g, nx, ny, nz, eps, r, gnorm2, phi, s);
     }
-    if (!xh || !xl) return cudaErrorInvalidValue;   // the FP32 path keeps the split copies
-    (phi ? tv_grad_split_kernel<true> : tv_grad_split_kernel<false>)<<<r.grid, kRedThreads, 0, s>>>(
+    if (!phi && (!xh || !xl)) return cudaErrorInvalidValue;   // the FP32 path keeps the split copies
+    (phi ? tv_grad_f32_kernel<true> : tv_grad_f32_kernel<false>)<<<r.grid, kRedThreads, 0, s>>>(
         x, xh, xl, (float*)g, nx, ny, nz, (float)eps, r.partials, r.ticket, gnorm2, phi);
     return cudaGetLastError();
 }

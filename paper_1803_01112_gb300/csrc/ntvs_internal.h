@@ -179,7 +179,7 @@ struct RedScratch {
 
 // The image x is always the FP64 master copy; g and the stencil arithmetic use cdt.
 // g = grad phi_eps(x); *gnorm2 = ||g||^2 (FP64); if phi != nullptr also *phi = phi_0(x).
-// On the FP32 path the stencil reads xh/xl instead of x (phi still comes from x).
+// On the FP32 path without phi the stencil reads xh/xl instead of x.
 cudaError_t k_tv_grad(int cdt, const double* x, const float* xh, const float* xl, void* g, int nx, int ny, int nz,
                       double eps, RedScratch r, double* gnorm2, double* phi, cudaStream_t s);
 // *phi = phi_0(z), z = x - sc*g with sc = beta/sqrt(*gnorm2) (z = x when g == nullptr or
