@@ -282,11 +282,25 @@ __global__ void otf_rows_kernel(const float* __restrict__ paths, int64_t M, Grid
 constexpr int kOtfThreads = 256;
 constexpr int kOtfWarps = kOtfThreads / 32;
 
-// entries of a warp's buffer: two rows of a straight path across the grid with its segment
-// joins, in 72 KB (three CTAs per SM) or, when that suffices, 54 KB (four) a CTA
-static int otf_buffer(const OtfArgs& a) {
+// Entries of a warp's buffer, from two rows' pieces on the grid's diagonal (every plane of x and y
+// crossed; straight in z) with their segment joins: 54 KB a CTA and four CTAs an SM, or 72 KB and
+// three, 114 KB and two, 225 KB and one.  Rows off the diagonal have fewer pieces (1.27 n on
+// average on n x n voxels, against 2 n), so a size serves grids somewhat past its diagonal; what
+// does not fit is walked twice, and slowest by far.  Sweeps of 400k rows of 16 segments with
+// three / two / one CTA, us (24 cached pieces a lane, before the buffer: last number):
+//   256x256x16  669 / 704 / 1099 (1088)     512x512x16  2410 / 1483 / 1878 (2379)
+//   320x320x16  913 / 837 / 1295 (1413)     576x576x16  3050 / 1962 / 2064 (2745)
+//   448x448x16  1837 / 1142 / 1691 (2059)   640x640x8   2945 / 2352 / 2092 (2833)
+//   1024x256x8  1886 / 1554 / 1666 (2019)   1024x1024x4 4566 / 4175 / 3253 (4302)
+struct OtfBuffer {
+    int entries, ctas;   // per warp; CTAs an SM
+};
+static OtfBuffer otf_buffer(const OtfArgs& a) {
     const int64_t need = 2 * ((int64_t)a.nx + a.ny + 2 * a.n_seg + 8);
-    return need <= 864 ? 864 : 1136;
+    if (need <= 864) return {864, 4};
+    if (need <= 1136) return {1136, 3};
+    if (need <= 2500) return {1776, 2};
+    return {3520, 1};
 }
 
 template <int MINB>
@@ -397,7 +411,8 @@ __global__ void __launch_bounds__(kOtfThreads, MINB) otf_drop_kernel(const float
 
 // ---------------------------------------------------------------- forward projection
 // out_i = sum of l * x_v over the accepted pieces (voxel v, length l >= min_len) of history
-// i's path, the rows the DROP sweeps use; 16 lanes per row, each tracing every 16th segment.
+// i's path, the stored rows' lengths (the DROP sweeps step their crossings and differ by about an
+// ulp of t in each); 16 lanes per row, each tracing every 16th segment.
 __global__ void __launch_bounds__(256) otf_project_kernel(const float* __restrict__ paths, int64_t M, Grid3 g,
                                                            int n_seg, float min_len, const float* __restrict__ x,
                                                            void* __restrict__ out, int out64) {
@@ -514,14 +529,14 @@ cudaError_t k_otf_prep(const OtfArgs& a, int64_t r0, int64_t r1, float* inv_norm
 cudaError_t k_otf_drop(const OtfArgs& a, int64_t r0, int64_t r1, const float* inv_norm2, const float* x, float* delta,
                        double lambda, double* resid_ss, cudaStream_t s) {
     if (r1 <= r0) return cudaSuccess;
-    const int cap = otf_buffer(a);
-    const size_t smem = (size_t)cap * kOtfWarps * sizeof(int2);
-    auto kern = cap == 864 ? otf_drop_kernel<4> : otf_drop_kernel<3>;
+    const OtfBuffer buf = otf_buffer(a);
+    const size_t smem = (size_t)buf.entries * kOtfWarps * sizeof(int2);
+    auto kern = buf.ctas == 4 ? otf_drop_kernel<4> : buf.ctas == 3 ? otf_drop_kernel<3> : otf_drop_kernel<2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int grid = a.grid / 8 * (cap == 864 ? 4 : 3);   // a.grid: 8 CTAs per SM; one resident wave
+    const int grid = a.grid / 8 * buf.ctas;   // a.grid: 8 CTAs per SM; one resident wave
     kern<<<grid < 1 ? 1 : grid, kOtfThreads, smem, s>>>(a.paths, a.b, inv_norm2, r0, r1, make_grid(a), a.n_seg, a.min_len, x, delta,
-                                           (float)lambda, resid_ss, cap);
+                                           (float)lambda, resid_ss, buf.entries);
     return cudaGetLastError();
 }
 
