@@ -81,7 +81,7 @@ struct MemberDev {
     double* resid;             // [B]
     WinStat* wstat;            // [B] statistics of the blocks' rows, and
     float* rms;                // the rms residual of the last swept block (the fixed-point DROP window's
-                               // scale, as in the single-context kernel)
+    float2* wsums;             // scale, as in the single-context kernel), and the current block's sums
     double* tv_hist;           // [cap]
     int nx, ny, nz, B, N;
     int64_t V;
@@ -383,7 +383,10 @@ __device__ void drop_rows(const MemberDev& m, int64_t i0, int64_t i1, int w0, in
         }
     }
     const double tot = block_sum(ss, sh);
-    if (threadIdx.x == 0 && tot != 0.0) atomicAdd(resid_b, tot);
+    if (threadIdx.x == 0 && tot != 0.0) {
+        atomicAdd(resid_b, tot);
+        asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(m.wsums), "f"(__log2f((float)tot)), "f"(1.f) : "memory");
+    }
 }
 
 __device__ void drop_item(const MemberDev& m, int b, int idx, int win_cap, double* sh) {
@@ -505,8 +508,8 @@ __device__ void finish_phase(const CycleArgs& a, int r, int phase, int items, un
             n += 1;
             break;
         case PH_DROP:   // the next block's window scale
-            *(volatile float*)m.rms =
-                (float)sqrt(*(volatile double*)(m.resid + b) / (double)(m.block_ptr[b + 1] - m.block_ptr[b]));
+            *(volatile float*)m.rms = win_rms(__ldcg(m.wsums), (float)(m.block_ptr[b + 1] - m.block_ptr[b]));
+            __stcg(m.wsums, make_float2(0.f, 0.f));
             ph = PH_DAPPLY;
             break;
         case PH_DAPPLY:
@@ -1042,9 +1045,10 @@ int member_prep(ntvs_batch* bt, ntvs_batch::Member& mm, const void* x0, int x0_d
     if (M > 0) norm_kernel<<<grid_of(M * 32), 256, 0, s>>>(d.row_ptr, d.val, M, (float*)d.inv_norm2);
     int32_t* cnt = nullptr;
     BTRY(balloc(&cnt, sizeof(int32_t) * VI, "hit counts"));
-    BTRY(member_alloc(mm, (void**)&d.wstat, sizeof(WinStat) * (size_t)B + sizeof(float), "window statistics"));
-    cudaMemsetAsync(d.wstat, 0, sizeof(WinStat) * (size_t)B, s);
-    d.rms = reinterpret_cast<float*>(d.wstat + B);
+    BTRY(member_alloc(mm, (void**)&d.wstat, sizeof(WinStat) * (size_t)B + sizeof(float2) + sizeof(float), "window statistics"));
+    d.wsums = reinterpret_cast<float2*>(d.wstat + B);
+    d.rms = reinterpret_cast<float*>(d.wsums + 1);
+    cudaMemsetAsync(d.wstat, 0, sizeof(WinStat) * (size_t)B + sizeof(float2), s);
     cudaMemsetAsync(d.rms, 0xff, sizeof(float), s);   // NaN: no residuals seen yet
     for (int t = 0; t < B; ++t) {
         cudaMemsetAsync(cnt, 0, sizeof(int32_t) * VI, s);

@@ -102,22 +102,31 @@ struct WinScale {
 };
 
 // The scale for a block whose rows have the statistics st (WinStat), rms being the root mean
-// square residual of the block swept before it (NaN: none, the image was set since).  The bound
-// is 10 rms on a row of mean ||a||^2, never below 1/16 and never above 4 of the block's mean |b|,
-// and 1/4 of it without an rms: so the quantum follows the residuals of the image being swept,
-// is at most 4 mean |b| coarse whatever an earlier sweep saw, and rows of very short chords, whose
-// |r / lambda| is far above the others', scatter globally instead of coarsening them.
-// At 10 rms the error of a sweep against 64 bits is that of FP32 reductions (2.773e-8 of the image
-// at 200x200x16, 2M rows in detected order, both ways); at 4 mean |b| it would be 2.9e-8.
+// square residual of the block swept before it (win_rms).  The bound on a row of mean ||a||^2 is
+// 10 rms, or 4 once the residuals are of the size of b itself (they are then mostly of one sign, not
+// noise), between 1/16 and 64 of the block's mean |b|; without an rms 1/4 of it (NaN: the image was
+// set since) or 4 (below 0: the zero image of a load, whose residual is b).  So the quantum follows
+// the residuals of the image being swept, and rows of very short chords, whose |r / lambda| is far
+// above the others', scatter globally instead of coarsening them.  At 10 rms the error of a sweep
+// against 64 bits is that of FP32 reductions (2.773e-8 of the image at 200x200x16, 2M rows in
+// detected order, both ways).
 // A scale taken inside the launch, from its own first rows, was exact about the image but cost 6
 // of 62 us a block of 100k rows (the other warps wait for it, or scatter globally until it stands).
 __device__ __forceinline__ WinScale win_scale(float lambda, const WinStat& st, float rms) {
-    float bound = rms >= 0.f ? 10.f * rms : 0.25f * st.mean_b;
-    if (st.mean_b > 0.f) bound = fminf(fmaxf(bound, 0.0625f * st.mean_b), 4.f * st.mean_b);
+    float bound = rms >= 0.f  ? fminf(10.f * rms, 4.f * fmaxf(rms, st.mean_b))
+                  : rms < 0.f ? 4.f * st.mean_b
+                              : 0.25f * st.mean_b;
+    if (st.mean_b > 0.f) bound = fminf(fmaxf(bound, 0.0625f * st.mean_b), 64.f * st.mean_b);
     bound *= st.inv_norm2;
     const float lam = fabsf(lambda), Q = lam * bound * st.lmax * 0x1p-30f, iq = 1.f / Q;
     if (!(st.amax > 0.f && Q > 0.f && isfinite(Q) && isfinite(iq))) return WinScale{0.f, 0.f, 0.f};
     return WinScale{iq, fminf(bound, 0x1p22f * Q / (lam * st.amax)), Q};
+}
+// The rms residual of a swept block of `rows` rows from the sums over its runs of rows (a CTA's each,
+// of about equal length): {sum of log2(residual sum of squares), runs with any}.  Their geometric
+// mean, which a few rows of corrupt data in a few runs hardly move.
+__device__ __forceinline__ float win_rms(float2 sums, float rows) {
+    return sums.y > 0.f ? exp2f(0.5f * (sums.x / sums.y - __log2f(rows / sums.y))) : 0.f;
 }
 
 // %globaltimer in nanoseconds (the clock of every bounded device-side wait)

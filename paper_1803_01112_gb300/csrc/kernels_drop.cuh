@@ -436,7 +436,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
                          const V* __restrict__ val, const T* __restrict__ b, const T* __restrict__ inv_norm2,
                          const DropSegment* __restrict__ segs, const int32_t* __restrict__ seg_begin,
                          int64_t slice, const T* __restrict__ x, T* __restrict__ delta, T lambda,
-                         double* resid_ss, Delta16 d16, const WinStat* wstat, const float* wrms,
+                         double* resid_ss, Delta16 d16, const WinStat* wstat, const float* wrms, bool wzero, float* wlog,
                          const int32_t* __restrict__ row_order) {
     static_assert(!ORD || (!D16 && sizeof(T) == 4 && 20 * kOrderedStage <= stage_bytes_all<float, false>()),
                   "ordered rows are packed FP32 pairs and stage in the space of the others");
@@ -451,7 +451,7 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
     const int nwarps = blockDim.x >> 5;
     for (int j = threadIdx.x; j < W; j += blockDim.x) win[j] = 0;
     for (int q = threadIdx.x; q < 32 * G; q += blockDim.x) (&ss_grp[0][0])[q] = 0.0;
-    if (threadIdx.x == 0) ws = win_scale((float)lambda, *wstat, *wrms);
+    if (threadIdx.x == 0) ws = win_scale((float)lambda, *wstat, wrms ? *wrms : wzero ? -1.f : __int_as_float(0x7fffffff));
     __syncthreads();
     const int s0 = seg_begin[blockIdx.x], s1 = seg_begin[blockIdx.x + 1];
     int cur = s0 < s1 ? segs[s0].home : 0;
@@ -535,7 +535,10 @@ drop_block_window_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __r
     if (lane < G) ss = ss_grp[warp][lane];
     __shared__ double sh[32];
     const double tot = block_sum(ss, sh);   // synchronizes the CTA
-    if (threadIdx.x == 0 && tot != 0.0) atomicAdd(resid_ss, tot);
+    if (threadIdx.x == 0) {
+        if (tot != 0.0) atomicAdd(resid_ss, tot);
+        wlog[blockIdx.x] = tot != 0.0 ? __log2f((float)tot) : INFINITY;
+    }
 }
 
 // ------------------------------------------------------------------ launch
@@ -547,7 +550,8 @@ cudaError_t launch_window(const DropArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     kern<<<a.grid, 1024, smem, s>>>(a.row_ptr, a.col, (const V*)a.val, (const T*)a.b, (const T*)a.inv_norm2, a.segs,
                                     a.seg_begin, a.slice, (const T*)a.x, (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16,
-                                    a.wstat, a.wrms, a.order);
+                                    a.wstat, a.wrms, a.wzero, a.wlog,
+                                    a.order);
     return cudaGetLastError();
 }
 

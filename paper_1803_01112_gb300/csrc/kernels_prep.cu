@@ -75,26 +75,28 @@ namespace ntvs {
 // row), and the hit counts of the entries with a != 0.  Requires a validated row_ptr.
 // FP64 path (cs null): cnt[j] += 1.
 // FP32 path (cs not null): cs[j] += {1, |a_ij|}, the hit count and the block's column sum of
-// lengths with one two-element reduction; st takes the largest |a_ij| (an atomic maximum of the
-// bits of non-negative floats) and the sums of ||a_i||^2 and |b_i|.  A count is
+// lengths with one two-element reduction, and *amax_out = max |a_ij| (as float bits, an atomic
+// maximum of non-negative floats): statistics of the fixed-point DROP window.  A count is
 // exact below 2^24, where it stays; finish_block_kernel reports it.
 // PACK (FP32 values in CSR32 storage): col holds canonical columns; entry p leaves as the pair
 // {internal column, value bits} in ent[p], so columns and values are read once and never
 // rewritten.  62M entries: 1375 us (bound by the reductions), against 285 + 1425 + 195 us for
 // remapping, this pass and packing one after the other, 40 bytes an entry instead of 16.
+// Registers for five CTAs an SM: left to itself the compiler fits six, and 25 000 rows of 132 entries
+// (20 blocks) took 72.4 us a block instead of 63.9.
 template <typename V, typename T, bool PACK>
-__global__ void __launch_bounds__(256) prep_block_kernel(const int64_t* __restrict__ row_ptr,
+__global__ void __launch_bounds__(256, 5) prep_block_kernel(const int64_t* __restrict__ row_ptr,
                                                          const int32_t* __restrict__ col, const V* __restrict__ val,
                                                          int64_t e0, const T* __restrict__ b, int64_t r0, int64_t r1,
                                                          int64_t nvox, VoxMap vm, T* __restrict__ inv_norm2,
                                                          int32_t* __restrict__ cnt, int* flags,
-                                                         float2* __restrict__ cs, WinStat* st,
+                                                         float2* __restrict__ cs, unsigned* amax_out,
                                                          int2* __restrict__ ent) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     int f = 0;
-    float amax = 0.f, asum = 0.f, bsum = 0.f;
+    float amax = 0.f;
     for (int64_t i = r0 + w0; i < r1; i += nw) {
         const int64_t p0 = __ldg(row_ptr + i), p1 = __ldg(row_ptr + i + 1);
         double sq = 0.0;
@@ -127,28 +129,20 @@ __global__ void __launch_bounds__(256) prep_block_kernel(const int64_t* __restri
             inv_norm2[i] = (T)inv;
             const double bi = (double)b[i];
             if (!isfinite(bi)) f |= 16;
-            asum += (float)sq;
-            bsum += (float)fabs(bi);
         }
     }
     if (f) atomicOr(flags, f);
-    if (st) {
+    if (amax_out) {
         for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        if (lane == 0 && amax > 0.f) atomicMax(reinterpret_cast<unsigned*>(&st->amax), __float_as_uint(amax));
-        if (lane == 0 && asum > 0.f) atomicAdd(&st->inv_norm2, asum);
-        if (lane == 0 && bsum > 0.f) atomicAdd(&st->mean_b, bsum);
+        if (lane == 0 && amax > 0.f) atomicMax(amax_out, __float_as_uint(amax));
     }
 }
 
 // A block's counts and column sums once its rows are through: inv_s[j] = 1 / count (0 for an
-// unhit voxel), st->lmax = max_j of the sums, and cs cleared for the next block; the row sums in st
-// become means; flags |= 64 when a count reached 2^24.
+// unhit voxel), st->lmax = max_j of the sums, and cs cleared for the next block; flags |= 64 when a
+// count reached 2^24.
 __global__ void __launch_bounds__(256) finish_block_kernel(float2* __restrict__ cs, int64_t n, float* __restrict__ inv_s,
-                                                           WinStat* st, float rows, int* flags) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        st->inv_norm2 = st->inv_norm2 > 0.f ? rows / st->inv_norm2 : 0.f;
-        st->mean_b /= rows;
-    }
+                                                           WinStat* st, int* flags) {
     float m = 0.f;
     bool full = false;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
@@ -163,12 +157,43 @@ __global__ void __launch_bounds__(256) finish_block_kernel(float2* __restrict__ 
     if (full) atomicOr(flags, 64);
 }
 
-cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, WinStat* st, int64_t rows, int* flags,
-                           cudaStream_t s) {
+cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, WinStat* st, int* flags, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int64_t need = (n + 255) / 256;
     const int grid = (int)(need < prep_grid() ? need : prep_grid());
-    finish_block_kernel<<<grid, 256, 0, s>>>(cs, n, inv_s, st, (float)(rows > 0 ? rows : 1), flags);
+    finish_block_kernel<<<grid, 256, 0, s>>>(cs, n, inv_s, st, flags);
+    return cudaGetLastError();
+}
+
+// A CTA per block: the means of ||a_i||^2 and |b_i| in st, over at most kStatRows of its rows, evenly
+// spaced (sums over all rows in the preparation pass took 3 of its 68 us per 25 000 rows)
+constexpr int kStatRows = 4096;
+
+__global__ void __launch_bounds__(1024) row_stat_kernel(const int64_t* __restrict__ bp, const float* __restrict__ b,
+                                                        const float* __restrict__ inv_norm2, WinStat* st) {
+    __shared__ double sh[32];
+    const int64_t r0 = bp[blockIdx.x], r1 = bp[blockIdx.x + 1], step = (r1 - r0 + kStatRows - 1) / kStatRows;
+    float a2 = 0.f, ab = 0.f, k = 0.f;
+#pragma unroll
+    for (int q = 0; q < kStatRows / 1024; ++q) {
+        const int64_t i = r0 + ((int64_t)q * 1024 + threadIdx.x) * step;
+        if (i < r1) {
+            const float inv = inv_norm2[i];
+            if (inv > 0.f) a2 += 1.f / inv;
+            ab += fabsf(b[i]);
+            k += 1.f;
+        }
+    }
+    const double sa = block_sum(a2, sh), sb = block_sum(ab, sh), sk = block_sum(k, sh);
+    if (threadIdx.x == 0) {
+        st[blockIdx.x].inv_norm2 = sa > 0.0 ? (float)(sk / sa) : 0.f;
+        st[blockIdx.x].mean_b = sk > 0.0 ? (float)(sb / sk) : 0.f;
+    }
+}
+
+cudaError_t k_row_stats(const int64_t* bp, int B, const float* b, const float* inv_norm2, WinStat* st, cudaStream_t s) {
+    if (B <= 0) return cudaSuccess;
+    row_stat_kernel<<<B, 1024, 0, s>>>(bp, b, inv_norm2, st);
     return cudaGetLastError();
 }
 
@@ -193,17 +218,18 @@ cudaError_t k_recount(const int64_t* row_ptr, int64_t r0, int64_t r1, const int3
 template <typename V, typename T, bool PACK>
 static cudaError_t launch_prep(const int64_t* rp, const int32_t* col, const void* val, int64_t e0, const void* b,
                                int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inn, int32_t* cnt,
-                               int* flags, float2* cs, WinStat* st, int32_t* ent, cudaStream_t s) {
+                               int* flags, float2* cs, float* amax, int32_t* ent, cudaStream_t s) {
     prep_block_kernel<V, T, PACK><<<prep_grid(), 256, 0, s>>>(rp, col, (const V*)val, e0, (const T*)b, r0, r1, nvox, vm,
-                                                             (T*)inn, cnt, flags, cs, st, reinterpret_cast<int2*>(ent));
+                                                             (T*)inn, cnt, flags, cs, reinterpret_cast<unsigned*>(amax),
+                                                             reinterpret_cast<int2*>(ent));
     return cudaGetLastError();
 }
 
 cudaError_t k_prep_block(const int64_t* row_ptr, const int32_t* col, const void* val, int64_t e0, int vdt,
                          const void* b, int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inv_norm2,
-                         int cdt, int32_t* cnt, int* flags, float2* cs, WinStat* st, int32_t* ent, cudaStream_t s) {
+                         int cdt, int32_t* cnt, int* flags, float2* cs, float* amax, int32_t* ent, cudaStream_t s) {
     if (r1 <= r0) return cudaSuccess;
-#define NTVS_PREP(V, T, P) launch_prep<V, T, P>(row_ptr, col, val, e0, b, r0, r1, nvox, vm, inv_norm2, cnt, flags, cs, st, ent, s)
+#define NTVS_PREP(V, T, P) launch_prep<V, T, P>(row_ptr, col, val, e0, b, r0, r1, nvox, vm, inv_norm2, cnt, flags, cs, amax, ent, s)
     if (cdt == F64) {
         if (vdt == F64) return NTVS_PREP(double, double, false);
         if (vdt == F32) return ent ? NTVS_PREP(float, double, true) : NTVS_PREP(float, double, false);

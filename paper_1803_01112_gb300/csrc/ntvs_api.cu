@@ -116,7 +116,10 @@ struct ntvs_ctx {
     int32_t* stage_begin = nullptr;    // [B][win_grid + 1]
     int win_grid = 0;
     WinStat* wstat = nullptr;          // FP32: [B] statistics of the blocks' rows (scale of the window)
-    float* wrms = nullptr;             // FP32: rms residual of the last swept block (NaN: none since set_image)
+    float* wlog = nullptr;             // FP32: [sms] log2 residual sums of the block being swept, by CTA, then
+                                       // the rms residual of the one before (scale of the window)
+    bool seen = false;                 // that residual is of the present image
+    bool zero = false;                 // the image is the zero image of a load
     int* derr = nullptr;               // device error word (bounded waits that ran out)
     // DELTA16 index storage (packed at load from the int32 columns)
     uint16_t* d16off = nullptr;        // [nnz] column - chunk base
@@ -218,7 +221,7 @@ struct ntvs_ctx {
         dev_free(seg_begin);
         dev_free(order);
         dev_free(wstat);
-        dev_free(wrms);
+        dev_free(wlog);
         dev_free(stages);
         dev_free(stage_begin);
         dev_free(d16off);
@@ -565,13 +568,15 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
     a.order = nullptr;
     a.slice = c->vm.slice_p;
     a.wstat = c->wstat ? c->wstat + t : nullptr;
-    a.wrms = c->wrms;
     a.max_row = t < (int)c->block_maxrow.size() ? c->block_maxrow[t] : (int64_t)1 << 40;
     if (whole && c->schedule == NTVS_SCHED_WINDOW && c->segs) {
         a.segs = c->segs;
         a.order = c->order;
         a.seg_begin = c->seg_begin + (size_t)t * (c->win_grid + 1);
         a.grid = c->win_grid;
+        a.wlog = c->wlog;
+        a.wrms = c->seen ? c->wlog + c->sms : nullptr;
+        a.wzero = c->zero;
     }
     if (whole && c->schedule == NTVS_SCHED_PIPELINE) {
         DropPipeArgs pa;
@@ -612,6 +617,7 @@ int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
     const bool split = t == c->B - 1;
     if (!resid_cleared) CUDA_TRY(cudaMemsetAsync(c->resid + t, 0, sizeof(double), c->stream));
     if (r1 <= r0 && !c->ar_fn) return NTVS_OK;
+    const bool windowed = r1 > r0 && c->schedule == NTVS_SCHED_WINDOW && c->segs;
     TRY(launch_drop_kernel(c, t, r0, r1, c->resid + t));
     if (c->ar_fn) {
         int rc = c->ar_fn(c->delta, c->vm.vint, c->cdt, (void*)c->stream, c->ar_user);
@@ -623,9 +629,11 @@ int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
     CUDA_TRY(timed_launch(c, KIND_APPLY, [&] {
         return k_drop_apply(c->cdt, c->x, c->copies(split), c->delta,
                             (const char*)c->inv_s + (size_t)t * c->vm.vint * c->csz(), c->V, c->apply_grid,
-                            c->resid + t, r1 - r0, r1 > r0 ? c->wrms : nullptr, c->stream);
+                            windowed ? c->wlog : nullptr, c->win_grid, r1 - r0,
+                            windowed ? c->wlog + c->sms : nullptr, c->stream);
     }));
     c->split_stale = !split;
+    if (windowed) c->seen = true;
     return NTVS_OK;
 }
 
@@ -1283,8 +1291,7 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     if (c->cdt == F32) {
         TRY(dev_alloc(&c->wstat, sizeof(WinStat) * (size_t)c->B, "window scale statistics"));
         CUDA_TRY(cudaMemsetAsync(c->wstat, 0, sizeof(WinStat) * (size_t)c->B, st));
-        TRY(dev_alloc(&c->wrms, sizeof(float), "rms residual"));
-        CUDA_TRY(cudaMemsetAsync(c->wrms, 0x7f, sizeof(float), st));   // 3.4e38: at x = 0 the residual is b
+        TRY(dev_alloc(&c->wlog, sizeof(float) * ((size_t)c->sms + 1), "window residuals"));
         TRY(dev_alloc(&cs, sizeof(float2) * (size_t)VI, "hit counts and column sums"));
         CUDA_TRY(cudaMemsetAsync(cs, 0, sizeof(float2) * (size_t)VI, st));
     } else {
@@ -1308,10 +1315,8 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
         }
         CUDA_TRY(k_prep_block(c->row_ptr, bc, bv, e0, c->vdt, c->b, bp[t], bp[t + 1], pack ? V : VI, c->vm,
                               c->inv_norm2, c->cdt, cnt ? cnt + (size_t)t * VI : nullptr, c->dflags, cs,
-                              cs ? c->wstat + t : nullptr, c->ent, st));
-        if (cs)
-            CUDA_TRY(k_finish_block(cs, VI, (float*)c->inv_s + (size_t)t * VI, c->wstat + t, bp[t + 1] - bp[t],
-                                    c->dflags, st));
+                              cs ? &c->wstat[t].amax : nullptr, c->ent, st));
+        if (cs) CUDA_TRY(k_finish_block(cs, VI, (float*)c->inv_s + (size_t)t * VI, c->wstat + t, c->dflags, st));
         if (ring) {   // the slot is free again: the block nslots on may be copied into it
             cudaEvent_t ev;
             CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -1320,12 +1325,17 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
             if (t + nslots < c->B) TRY(issue_copy(t + nslots));
         }
     }
-    {   // longest row of every block
+    {   // longest row of every block, and the row statistics of the window's scale
         unsigned long long* dm = nullptr;
-        TRY(dev_alloc(&dm, sizeof(unsigned long long) * (size_t)c->B, "row lengths"));
+        TRY(dev_alloc(&dm, sizeof(unsigned long long) * (2 * (size_t)c->B + 1), "row lengths"));
         std::vector<unsigned long long> hm((size_t)c->B, 0);
         cudaError_t e = cudaMemsetAsync(dm, 0, sizeof(unsigned long long) * (size_t)c->B, st);
         for (int t = 0; t < c->B && e == cudaSuccess; ++t) e = k_row_maxlen(c->row_ptr, bp[t], bp[t + 1], dm + t, c->sms * 4, st);
+        int64_t* dbp = reinterpret_cast<int64_t*>(dm + c->B);
+        if (e == cudaSuccess && c->wstat)
+            e = cudaMemcpyAsync(dbp, bp.data(), sizeof(int64_t) * ((size_t)c->B + 1), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess && c->wstat)
+            e = k_row_stats(dbp, c->B, (const float*)c->b, (const float*)c->inv_norm2, c->wstat, st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(hm.data(), dm, sizeof(unsigned long long) * (size_t)c->B, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1411,6 +1421,8 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
     c->ar_user = nullptr;
     CUDA_TRY(cudaStreamSynchronize(st));
     c->split_stale = false;
+    c->seen = false;
+    c->zero = true;
     c->loaded = true;
     return NTVS_OK;
 }
@@ -1625,7 +1637,7 @@ int ntvs_set_image(ntvs_ctx* c, const void* x, int dtype, int mem_kind) {
         CUDA_TRY(cudaStreamSynchronize(c->stream));
     }
     if (c->x32) CUDA_TRY(k_x32_from_x64(c->x, c->copies(), c->stream));
-    if (c->wrms) CUDA_TRY(cudaMemsetAsync(c->wrms, 0xff, sizeof(float), c->stream));   // NaN: no residuals seen yet
+    c->seen = c->zero = false;
     c->split_stale = false;
     return NTVS_OK;
 }

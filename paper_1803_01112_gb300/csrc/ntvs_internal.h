@@ -14,15 +14,6 @@ enum Dt { F64 = 0, F32 = 1, F16 = 2, BF16 = 3 };
 
 inline size_t dt_size(int dt) { return dt == F64 ? 8 : dt == F32 ? 4 : 2; }
 
-// Internal voxel order of the FP32 gather copy, delta, hit counts and matrix columns:
-// in-plane tiles of tx x ty voxels, each tile contiguous, tiles row-major over a grid padded
-// to multiples of the tile, slices contiguous (slice_p voxels each).  With sw set, the
-// in-slice offset p of that order is stored at p ^ ((p >> 5) & 31): a bijection inside
-// each aligned group of 32 offsets (slice_p is then a multiple of 32), which is the bank
-// spread of the DROP kernels' slice windows, so that their window slot is the voxel's
-// offset in its slice.  tx = ty = 1 without sw is the canonical order (iz*ny + iy)*nx + ix.
-// Public images and the FP64 master stay canonical.  tx, ty are powers of two (ltx, lty
-// their logarithms); V and vint stay below 2^31.
 // u / d for u < 2^31 as a multiply and a shift: m = floor(2^(31+l) / d) + 1 with
 // l = ceil(log2 d) exceeds 2^(31+l) / d by less than 2^l / d, so u m / 2^(31+l) never reaches
 // the next integer; d = 1 keeps m = 0.
@@ -39,6 +30,15 @@ inline FastDiv make_fastdiv(uint32_t d) {
     return f;
 }
 
+// Internal voxel order of the FP32 gather copy, delta, hit counts and matrix columns:
+// in-plane tiles of tx x ty voxels, each tile contiguous, tiles row-major over a grid padded
+// to multiples of the tile, slices contiguous (slice_p voxels each).  With sw set, the
+// in-slice offset p of that order is stored at p ^ ((p >> 5) & 31): a bijection inside
+// each aligned group of 32 offsets (slice_p is then a multiple of 32), which is the bank
+// spread of the DROP kernels' slice windows, so that their window slot is the voxel's
+// offset in its slice.  tx = ty = 1 without sw is the canonical order (iz*ny + iy)*nx + ix.
+// Public images and the FP64 master stay canonical.  tx, ty are powers of two (ltx, lty
+// their logarithms); V and vint stay below 2^31.
 struct VoxMap {
     int nx, ny, nz;
     int nxp, nyp;      // padded to multiples of tx, ty
@@ -106,26 +106,26 @@ int red_grid(int64_t n, int sm_count);
 struct WinStat {
     float lmax;        // largest column sum of |a_ij|
     float amax;        // largest |a_ij|
-    float inv_norm2;   // rows / sum of ||a_i||^2 (while the block is prepared: the sum)
-    float mean_b;      // mean |b_i| (while the block is prepared: the sum)
+    float inv_norm2;   // 1 / mean ||a_i||^2
+    float mean_b;      // mean |b_i|
 };
-
 // flags |= 1 if row_ptr decreases, 2 if row_ptr[0] != 0
 cudaError_t k_validate_rows(const int64_t* row_ptr, int64_t M, int* flags, cudaStream_t s);
 // fused pass over the rows [r0, r1) of one block: validation of columns (against [0, nvox)),
 // values and b (flags 4 / 8 / 16), inv_norm2 of the rows and the block's hit counts: cnt[j] += 1,
-// or with cs (FP32 path) cs[j] += {1, |a_ij|} and *st takes the block's largest |a_ij| and the sums
-// of ||a_i||^2 and |b_i|.  col and val hold the entries from e0 on: entry p is
-// col[p - e0] (0 for whole arrays, the block's first entry for a staging slot).  With ent (FP32
+// or with cs (FP32 path) cs[j] += {1, |a_ij|} and *amax = max(*amax, max |a_ij|).  col and val hold
+// the entries from e0 on: entry p is col[p - e0] (0 for whole arrays, the block's first entry for a
+// staging slot).  With ent (FP32
 // values in CSR32 storage) col is canonical and entry p is also packed into pair p of ent, its
 // column in the order of vm; without it col is in that order already.
 cudaError_t k_prep_block(const int64_t* row_ptr, const int32_t* col, const void* val, int64_t e0, int vdt,
                          const void* b, int64_t r0, int64_t r1, int64_t nvox, const VoxMap& vm, void* inv_norm2,
-                         int cdt, int32_t* cnt, int* flags, float2* cs, WinStat* st, int32_t* ent, cudaStream_t s);
-// inv_s = 1 / hit count from cs, st->lmax = the largest column sum, st's sums over the block's rows
-// turned into means, cs cleared; flags |= 64 when a count reached 2^24 (recount then)
-cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, WinStat* st, int64_t rows, int* flags,
-                           cudaStream_t s);
+                         int cdt, int32_t* cnt, int* flags, float2* cs, float* amax, int32_t* ent, cudaStream_t s);
+// inv_s = 1 / hit count from cs, st->lmax = the largest column sum, cs cleared; flags |= 64 when a
+// count reached 2^24 (recount then)
+cudaError_t k_finish_block(float2* cs, int64_t n, float* inv_s, WinStat* st, int* flags, cudaStream_t s);
+// the means of ||a_i||^2 and |b_i| over the rows [bp[t], bp[t+1]) of each of the B blocks, in st[t]
+cudaError_t k_row_stats(const int64_t* bp, int B, const float* b, const float* inv_norm2, WinStat* st, cudaStream_t s);
 // cnt[j] += hits of the packed entries of rows [r0, r1)
 cudaError_t k_recount(const int64_t* row_ptr, int64_t r0, int64_t r1, const int32_t* ent, int32_t* cnt, cudaStream_t s);
 // col_out[p] = internal index of voxel col_in[p]; flags |= 4 for a column outside [0, V)
@@ -232,7 +232,9 @@ struct DropArgs {
     // FP32 windowed schedule: the window accumulates in int32 fixed point; its scale comes from the
     // block's statistics and the rms residual of the block swept before (WinScale)
     const WinStat* wstat;
-    const float* wrms;
+    const float* wrms;        // that residual; null: none since the image was set, or (wzero) since the
+    bool wzero;               // load, the image being zero
+    float* wlog;              // this block's: log2 of every CTA's residual sum of squares (+inf: none)
     int64_t max_row;      // longest row of the block (register steps of the windowed kernel)
 };
 // dynamic shared memory of the windowed DROP kernel for a slice of `slice` voxels
@@ -284,10 +286,10 @@ cudaError_t k_row_home(const int64_t* row_ptr, const int32_t* col, int stride, i
 cudaError_t k_chunk_home(const int32_t* home, const int64_t* chunk_start, int64_t nchunks, int32_t* out,
                          unsigned long long* changes, int grid, cudaStream_t s);
 // x_j += delta_p * inv_s_p on the FP64 master (p the internal index of j) and its FP32
-// copies; delta_p = 0.  With rms not null also *rms = sqrt(*resid_ss / rows), the block's root mean
-// square residual.
+// copies; delta_p = 0.  With wlog not null (the windowed launch's, ctas of them) also *rms = the block's rms
+// residual over its `rows` rows, by a CTA of its own.
 cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const void* inv_s, int64_t V, int grid,
-                         const double* resid_ss, int64_t rows, float* rms, cudaStream_t s);
+                         const float* wlog, int ctas, int64_t rows, float* rms, cudaStream_t s);
 
 // TMA-fed pipeline (drop_pipe_kernel): a stage is a run of at most kStageRows whole rows
 // of one home slice whose entries [e0, e0 + nent) fit one ring slot (e0 and nent aligned

@@ -139,3 +139,34 @@ def test_batch_scale_follows_its_rows(window):
     for _ in range(2):
         x, _ = oracle.drop_sweep(rp, col, val.astype(np.float64), b.astype(np.float64), np.array([0, M], np.int64), x, 1.0)
     assert rel_l2(zero, x) <= 1e-6
+
+
+@pytest.mark.parametrize("factor", [1e2, 1e6])
+@pytest.mark.parametrize("nx,nz,n_hist,unordered", [(40, 4, 40_000, False), (96, 7, 115_011, True)])
+def test_a_corrupt_measurement_does_not_coarsen_the_others(nx, nz, n_hist, unordered, factor):
+    """One right-hand side far off moves the voxels of its row; the others keep their precision, in the
+    sweep itself and in the next block's (whose scale follows the first one's residuals)."""
+    ntvs = ntvs_module()
+    s, rp, col, val, _, b = _system(nx, nz, n_hist, unordered, "f32")
+    bad = s.M // 5
+    b[bad] *= factor
+    bp = np.array([0, s.M // 2, s.M] if not unordered else [0, s.M], np.int64)
+    x0 = s.xstar * 0.9 + 0.05
+    want, _ = oracle.drop_sweep(rp, col, val.astype(np.float64), b.astype(np.float64), bp, x0, 1.1)
+    # what the bad row moved, directly or through rows that share its voxels, is not compared
+    b2 = b.copy()
+    b2[bad] /= factor
+    clean, _ = oracle.drop_sweep(rp, col, val.astype(np.float64), b2.astype(np.float64), bp, x0, 1.1)
+    other = np.abs(want - clean) <= 1e-3
+    assert other.mean() > 0.05
+    r = ntvs.Reconstructor(0)
+    try:
+        r.load((nx, nx, nz), rp, col, val, b, block_ptr=bp)
+        assert r.stats()["drop_schedule"] == NTVS_SCHED_WINDOW
+        r.set_params(lam=1.1, N=0, alpha=0.5)
+        for _ in range(2):
+            r.set_image(x0)
+            r.drop_sweep()
+            assert rel_l2(r.get_image()[other], want[other]) <= 1e-6
+    finally:
+        r.close()
