@@ -106,22 +106,28 @@ cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const voi
 // (packed pairs for FP32 values) or DELTA16 storage (words for 16-bit values); accumulated in
 // the compute type T, written as double when out64 is set, else as float.
 //
-// A warp takes 8 consecutive rows: their extents come with one load and their results leave
+// A warp takes up to 8 consecutive rows: their extents come with one load and their results leave
 // with one (row by row, a warp a row, each result was a 4-byte write to a sector of its own), and
 // while a row is summed the next one's lines are on their way to L2.  Up to 8 entries a lane
 // are loaded before their gathers, summed in the order of the entries.  2M rows of 255 FP32
 // pairs: 816 us with one row and one entry at a time, 684 us (0.94 of the measured copy rate).
+// Fewer rows than 8 for every warp of the grid go fewer to a warp, so that no warp idles (FEW: the
+// number at run time, and the lines of a long row asked of L2 four runs of entries ahead, as its
+// warp has no next row to wait behind).  A call on 5000 FP64 rows of 2000 entries took 485 us with 8
+// rows a warp and takes 70 so, on 100 rows of 100 000 FP32 pairs 8020 and 476.
 constexpr int kProjRows = 8, kProjStep = 8;
 
-template <typename T, typename V, bool D16>
+template <typename T, typename V, bool D16, bool FEW>
 __global__ void __launch_bounds__(256)
 project_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, Delta16 d16,
-               const V* __restrict__ val, int64_t M, const T* __restrict__ x, void* __restrict__ out, int out64) {
+               const V* __restrict__ val, int64_t M, int few, const T* __restrict__ x, void* __restrict__ out,
+               int out64) {
+    const int rows = FEW ? few : kProjRows;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t base = w0 * kProjRows; base < M; base += nw * kProjRows) {
-        const int n = (int)min((int64_t)kProjRows, M - base);
+    for (int64_t base = w0 * rows; base < M; base += nw * rows) {
+        const int n = (int)min((int64_t)rows, M - base);
         const int64_t rp = lane <= n ? __ldg(row_ptr + base + lane) : 0;
         T mine = (T)0;
         for (int r = 0; r < n; ++r) {
@@ -133,6 +139,11 @@ project_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
             const int32_t* cbr = D16 ? d16.cbase + (p0 >> 5) + base + r : nullptr;
             T acc = (T)0;
             for (int64_t p = p0 + lane; p < p1; p += 32 * kProjStep) {
+                if constexpr (FEW && packed_entries<V, D16>()) {
+                    const int64_t q = p - lane + 4 * 32 * kProjStep + 16 * lane;
+                    if (lane < 2 * kProjStep && q < p1)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const int2*>(col) + q));
+                }
                 int32_t c[kProjStep];
                 T a[kProjStep];
 #pragma unroll
@@ -166,14 +177,15 @@ project_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
 
 template <typename T, typename V>
 static cudaError_t launch_project(const DropArgs& a, int64_t M, const void* x, void* out, int out64, cudaStream_t s) {
-    const int64_t need = (M + 8 * kProjRows - 1) / (8 * kProjRows);   // 8 warps a CTA
+    const int64_t warps = (int64_t)a.grid * 8;   // 8 a CTA
+    const int64_t each = (M + warps - 1) / warps;
+    const int rows = (int)(each < kProjRows ? each : kProjRows);
+    const int64_t need = (M + 8 * rows - 1) / (8 * rows);
     const int grid = (int)(need < a.grid ? need : a.grid);
-    if (a.use_d16)
-        project_kernel<T, V, true><<<grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M, (const T*)x, out,
-                                                        out64);
-    else
-        project_kernel<T, V, false><<<grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M, (const T*)x,
-                                                         out, out64);
+    const bool few = rows < kProjRows;
+    const auto kern = a.use_d16 ? (few ? project_kernel<T, V, true, true> : project_kernel<T, V, true, false>)
+                                : (few ? project_kernel<T, V, false, true> : project_kernel<T, V, false, false>);
+    kern<<<grid, 256, 0, s>>>(a.row_ptr, a.col, a.d16, (const V*)a.val, M, rows, (const T*)x, out, out64);
     return cudaGetLastError();
 }
 
