@@ -3,6 +3,8 @@
 // local variations, introduced in Sec. II).  Forward differences on index spacing, zero past the last
 // index.  The image is tiny next to the system matrix (V floats), so these kernels live
 // in L2; every reduction is FP64 with a fixed reduction order (deterministic).
+#include <algorithm>
+
 #include "common.cuh"
 #include "voxel_coords.cuh"
 
@@ -33,7 +35,7 @@ struct Quotients {
     }
 };
 
-// FP64 path: grad phi_eps on tiles of 31 x (TY - 1) voxels, marching along z:
+// FP64 path, images that fill them: grad phi_eps on tiles of 31 x (TY - 1) voxels, marching along z:
 //   g_q = -sum_a d_a(q) / D_q + sum_{a: q-e_a inside} d_a(q-e_a) / D_{q-e_a}
 // with d_a(c) = x_{c+e_a} - x_c (0 past the last index) and D_c = sqrt(eps + |d(c)|^2).
 // Every voxel of the tile and of its low halo forms its three quotients d_a / D once; the x and
@@ -108,21 +110,22 @@ tv_grad_tile_kernel(const double* __restrict__ x, double* __restrict__ g, int nx
     }
 }
 
-// FP32 path, one thread per voxel: neighbour differences as FP32 numbers, the rest of the stencil
-// in FP32, ||g||^2 accumulated in FP64.  Without PHI every difference is (xh_a - xh_b) +
-// (xl_a - xl_b) from the split copies of the master image, so the stencil runs without FP64
-// arithmetic.  PHI: also phi_0(x), whose differences are formed in FP64 from the master image; the
-// gradient's are those, rounded once (128x128x16: 31.8 us so and 28.6 with the split ones, which
-// lose what xl has no bits for, 2^-49 of the voxel).
-template <bool PHI>
+// One thread per voxel (the FP32 path, and FP64 images too thin for tiles).  SPLIT (FP32): neighbour
+// differences are (xh_a - xh_b) + (xl_a - xl_b) from the split copies of the master image, so the
+// stencil runs without FP64 arithmetic (only ||g||^2 is accumulated in FP64).  Otherwise they are
+// formed in FP64 from the master image and rounded once to T, the stencil's type; with PHI also
+// phi_0(x), from the same differences (FP32 on 128x128x16: 31.8 us so and 28.6 with the split ones,
+// which lose what xl has no bits for, 2^-49 of the voxel).
+template <typename T, bool SPLIT, bool PHI>
 __global__ void __launch_bounds__(kRedThreads)
-tv_grad_f32_kernel(const double* __restrict__ x, const float* __restrict__ xh, const float* __restrict__ xl,
-                   float* __restrict__ g, int nx, int ny, int nz, float eps, double* partials, unsigned* ticket,
-                   double* gnorm2, double* phi) {
+tv_grad_voxel_kernel(const double* __restrict__ x, const float* __restrict__ xh, const float* __restrict__ xl,
+                     T* __restrict__ g, int nx, int ny, int nz, T eps, double* partials, unsigned* ticket,
+                     double* gnorm2, double* phi) {
+    static_assert(!(SPLIT && PHI), "phi takes the differences of the master image");
     const int64_t sxy = (int64_t)nx * ny, V = sxy * nz;
-    auto dif = [&](int64_t a, int64_t b) -> float {
-        if constexpr (PHI) return (float)(__ldg(x + a) - __ldg(x + b));
-        else return (__ldg(xh + a) - __ldg(xh + b)) + (__ldg(xl + a) - __ldg(xl + b));
+    auto dif = [&](int64_t a, int64_t b) -> T {
+        if constexpr (SPLIT) return (__ldg(xh + a) - __ldg(xh + b)) + (__ldg(xl + a) - __ldg(xl + b));
+        else return (T)(__ldg(x + a) - __ldg(x + b));
     };
     double acc[PHI ? 2 : 1] = {};
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < V; p += (int64_t)gridDim.x * blockDim.x) {
@@ -130,35 +133,35 @@ tv_grad_f32_kernel(const double* __restrict__ x, const float* __restrict__ xh, c
         voxel_coords(p, nx, ny, ix, iy, iz);
         const bool hx = ix + 1 < nx, hy = iy + 1 < ny, hz = iz + 1 < nz;
         double ex = 0.0, ey = 0.0, ez = 0.0;
-        float dx, dy, dz;
+        T dx, dy, dz;
         if constexpr (PHI) {
             const double xc = __ldg(x + p);
             ex = hx ? __ldg(x + p + 1) - xc : 0.0;
             ey = hy ? __ldg(x + p + nx) - xc : 0.0;
             ez = hz ? __ldg(x + p + sxy) - xc : 0.0;
-            dx = (float)ex, dy = (float)ey, dz = (float)ez;
+            dx = (T)ex, dy = (T)ey, dz = (T)ez;
         } else {
-            dx = hx ? dif(p + 1, p) : 0.f, dy = hy ? dif(p + nx, p) : 0.f, dz = hz ? dif(p + sxy, p) : 0.f;
+            dx = hx ? dif(p + 1, p) : (T)0, dy = hy ? dif(p + nx, p) : (T)0, dz = hz ? dif(p + sxy, p) : (T)0;
         }
-        const float D = sqrtf(eps + (dx * dx + dy * dy + dz * dz));
-        float gq = (D > 0.f) ? -(dx + dy + dz) / D : 0.f;
+        const T D = sqrt(eps + (dx * dx + dy * dy + dz * dz));
+        T gq = (D > (T)0) ? -(dx + dy + dz) / D : (T)0;
         if (ix > 0) {
             const int64_t q = p - 1;
-            const float a = dif(p, q), b = hy ? dif(q + nx, q) : 0.f, c = hz ? dif(q + sxy, q) : 0.f;
-            const float Dm = sqrtf(eps + (a * a + b * b + c * c));
-            if (Dm > 0.f) gq += a / Dm;
+            const T a = dif(p, q), b = hy ? dif(q + nx, q) : (T)0, c = hz ? dif(q + sxy, q) : (T)0;
+            const T Dm = sqrt(eps + (a * a + b * b + c * c));
+            if (Dm > (T)0) gq += a / Dm;
         }
         if (iy > 0) {
             const int64_t q = p - nx;
-            const float a = dif(p, q), b = hx ? dif(q + 1, q) : 0.f, c = hz ? dif(q + sxy, q) : 0.f;
-            const float Dm = sqrtf(eps + (a * a + b * b + c * c));
-            if (Dm > 0.f) gq += a / Dm;
+            const T a = dif(p, q), b = hx ? dif(q + 1, q) : (T)0, c = hz ? dif(q + sxy, q) : (T)0;
+            const T Dm = sqrt(eps + (a * a + b * b + c * c));
+            if (Dm > (T)0) gq += a / Dm;
         }
         if (iz > 0) {
             const int64_t q = p - sxy;
-            const float a = dif(p, q), b = hx ? dif(q + 1, q) : 0.f, c = hy ? dif(q + nx, q) : 0.f;
-            const float Dm = sqrtf(eps + (a * a + b * b + c * c));
-            if (Dm > 0.f) gq += a / Dm;
+            const T a = dif(p, q), b = hx ? dif(q + 1, q) : (T)0, c = hy ? dif(q + nx, q) : (T)0;
+            const T Dm = sqrt(eps + (a * a + b * b + c * c));
+            if (Dm > (T)0) gq += a / Dm;
         }
         g[p] = gq;
         acc[0] += (double)gq * (double)gq;
@@ -270,11 +273,15 @@ static int sm_count() {
     return g_sm_count;
 }
 
+static int64_t grad_tiles(int nx, int ny, int ty) {
+    return (int64_t)((nx + kGradTx - 2) / (kGradTx - 1)) * ((ny + ty - 2) / (ty - 1));
+}
+
 template <bool PHI, int kGradTy>
 static cudaError_t launch_grad_tile(const double* x, double* g, int nx, int ny, int nz, double eps, RedScratch r,
                                     double* gnorm2, double* phi, cudaStream_t s) {
-    const int tiles_x = (nx + kGradTx - 2) / (kGradTx - 1), tiles_y = (ny + kGradTy - 2) / (kGradTy - 1);
-    const int64_t tiles = (int64_t)tiles_x * tiles_y;
+    const int tiles_x = (nx + kGradTx - 2) / (kGradTx - 1);
+    const int64_t tiles = grad_tiles(nx, ny, kGradTy);
     const int sms = sm_count();
     // slices per CTA: the fewest slice steps (a slice of halo each) on the busiest SM
     int zc = 1;
@@ -296,14 +303,26 @@ static cudaError_t launch_grad_tile(const double* x, double* g, int nx, int ny, 
 cudaError_t k_tv_grad(int cdt, const double* x, const float* xh, const float* xl, void* g, int nx, int ny, int nz,
                       double eps, RedScratch r, double* gnorm2, double* phi, cudaStream_t s) {
     if (cdt == F64) {
-        const bool few = (int64_t)nx * ny * nz < (int64_t)sm_count() * kGradTx * 16;   // under a tile slice an SM
+        const int64_t V = (int64_t)nx * ny * nz, slice = (int64_t)sm_count() * kGradTx * 16;   // a tile slice an SM
+        const bool few = V < slice;
+        // A voxel costs twice as much FP64 work by itself as in a tile, where every thread does it, inside the
+        // image or not: tiles as long as their threads are less than twice the voxels, or all run
+        // at once.  A step on 1x2000x50 voxels takes 256 us in tiles and 29 without, on 1x1x100000
+        // 2253 and 23; on 33x33x200, where tiles would have 2.6 threads a voxel, 59 without (73 before
+        // tiles).
+        const int64_t threads = grad_tiles(nx, ny, few ? 4 : 16) * nz * kGradTx * (few ? 4 : 16);
+        if (threads > std::max(2 * V, slice)) {
+            const auto kern = phi ? tv_grad_voxel_kernel<double, false, true> : tv_grad_voxel_kernel<double, false, false>;
+            kern<<<r.grid, kRedThreads, 0, s>>>(x, xh, xl, (double*)g, nx, ny, nz, eps, r.partials, r.ticket, gnorm2, phi);
+            return cudaGetLastError();
+        }
         const auto run = few ? (phi ? launch_grad_tile<true, 4> : launch_grad_tile<false, 4>)
                              : (phi ? launch_grad_tile<true, 16> : launch_grad_tile<false, 16>);
         return run(x, (double*)g, nx, ny, nz, eps, r, gnorm2, phi, s);
     }
     if (!phi && (!xh || !xl)) return cudaErrorInvalidValue;   // the FP32 path keeps the split copies
-    (phi ? tv_grad_f32_kernel<true> : tv_grad_f32_kernel<false>)<<<r.grid, kRedThreads, 0, s>>>(
-        x, xh, xl, (float*)g, nx, ny, nz, (float)eps, r.partials, r.ticket, gnorm2, phi);
+    const auto kern = phi ? tv_grad_voxel_kernel<float, false, true> : tv_grad_voxel_kernel<float, true, false>;
+    kern<<<r.grid, kRedThreads, 0, s>>>(x, xh, xl, (float*)g, nx, ny, nz, (float)eps, r.partials, r.ticket, gnorm2, phi);
     return cudaGetLastError();
 }
 
