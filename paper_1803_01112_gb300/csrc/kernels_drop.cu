@@ -68,6 +68,33 @@ __global__ void __launch_bounds__(256) drop_apply_kernel(double* __restrict__ x,
     }
 }
 
+// A thread per voxel; the copies' loads go out together, eight at a time.
+__global__ void __launch_bounds__(256) drop_apply_copies_kernel(double* __restrict__ x, double* __restrict__ delta,
+                                                                int copies, int64_t stride,
+                                                                const double* __restrict__ inv_s, int64_t V) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= V) return;
+    double d = 0.0;
+    for (int r0 = 0; r0 < copies; r0 += 8) {
+        double v[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = r0 + r < copies ? delta[(r0 + r) * stride + j] : 0.0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            d += v[r];
+            if (v[r] != 0.0) delta[(r0 + r) * stride + j] = 0.0;
+        }
+    }
+    if (d != 0.0) x[j] += d * __ldg(inv_s + j);
+}
+
+cudaError_t k_drop_apply_copies(double* x, double* delta, int copies, int64_t delta_stride, const double* inv_s,
+                                int64_t V, cudaStream_t s) {
+    if (V <= 0) return cudaSuccess;
+    drop_apply_copies_kernel<<<(unsigned)((V + 255) / 256), 256, 0, s>>>(x, delta, copies, delta_stride, inv_s, V);
+    return cudaGetLastError();
+}
+
 int64_t k_window_smem_bytes(int64_t slice, int csz, bool d16) {
     return (int64_t)window_smem_bytes(slice, (size_t)csz, d16);
 }

@@ -370,11 +370,15 @@ __device__ __forceinline__ void drop_row_any(int64_t i, const RowHead& h, bool v
 }
 
 // Plain variant: grid-stride over the rows of the block.
-template <typename T, typename V, int LPR, int CH, int VW, bool D16>
+// COPIES (FP64): CTA c scatters into copy c % copies of delta.  A form of its own, since the offset costs
+// the others registers (80 -> 110).
+template <typename T, typename V, int LPR, int CH, int VW, bool D16, bool COPIES = false>
 __global__ void __launch_bounds__(256)
 drop_block_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, const V* __restrict__ val,
                   const T* __restrict__ b, const T* __restrict__ inv_norm2, int64_t r0, int64_t r1,
-                  const T* __restrict__ x, T* __restrict__ delta, T lambda, double* resid_ss, Delta16 d16) {
+                  const T* __restrict__ x, T* __restrict__ delta, T lambda, double* resid_ss, Delta16 d16, int copies,
+                  int64_t delta_stride) {
+    if constexpr (COPIES) delta += (int64_t)(blockIdx.x % copies) * delta_stride;
     constexpr int G = 32 / LPR;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -568,9 +572,12 @@ static cudaError_t launch_cfg(const DropArgs& a, cudaStream_t s) {
     // slice the 1216 CTAs of a large block, nearly all without a row, took 8.5 us against 5.3
     const int64_t need = (a.r1 - a.r0 + 8 * (32 / LPR) - 1) / (8 * (32 / LPR));
     const int grid = (int)(need < a.grid ? need : a.grid);
-    drop_block_kernel<T, V, LPR, CH, VW, D16><<<grid, 256, 0, s>>>(
+    auto kern = drop_block_kernel<T, V, LPR, CH, VW, D16>;
+    if constexpr (sizeof(T) == 8)
+        if (a.copies > 1) kern = drop_block_kernel<T, V, LPR, CH, VW, D16, true>;
+    kern<<<grid, 256, 0, s>>>(
         a.row_ptr, a.col, (const V*)a.val, (const T*)a.b, (const T*)a.inv_norm2, a.r0, a.r1, (const T*)a.x,
-        (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16);
+        (T*)a.delta, (T)a.lambda, a.resid_ss, a.d16, a.copies, a.delta_stride);
     return cudaGetLastError();
 }
 

@@ -305,13 +305,13 @@ cudaError_t k_tv_grad(int cdt, const double* x, const float* xh, const float* xl
     if (cdt == F64) {
         const int64_t V = (int64_t)nx * ny * nz, slice = (int64_t)sm_count() * kGradTx * 16;   // a tile slice an SM
         const bool few = V < slice;
-        // A voxel costs twice as much FP64 work by itself as in a tile, where every thread does it, inside the
-        // image or not: tiles as long as their threads are less than twice the voxels, or all run
-        // at once.  A step on 1x2000x50 voxels takes 256 us in tiles and 29 without, on 1x1x100000
-        // 2253 and 23; on 33x33x200, where tiles would have 2.6 threads a voxel, 59 without (73 before
-        // tiles).
+        // In tiles every thread does a voxel's work, inside the image or not; by itself a voxel costs more
+        // than twice as much.  So tiles as long as they have at most three threads a voxel, or all run at
+        // once.  us a step in tiles / without, by threads a voxel: 63x33x64 (2.2) 35 / 41, 33x33x200 (2.8)
+        // 56 / 59, 31x5x3000 (3.3) 90 / 103, 34x18x128 (3.3) 33 / 31, 16x16x400 (4.0) 43 / 33, 400x2x200 (5)
+        // 82 / 47, 1x2000x50 (17) 256 / 29.
         const int64_t threads = grad_tiles(nx, ny, few ? 4 : 16) * nz * kGradTx * (few ? 4 : 16);
-        if (threads > std::max(2 * V, slice)) {
+        if (threads > std::max(3 * V, slice)) {
             const auto kern = phi ? tv_grad_voxel_kernel<double, false, true> : tv_grad_voxel_kernel<double, false, false>;
             kern<<<r.grid, kRedThreads, 0, s>>>(x, xh, xl, (double*)g, nx, ny, nz, eps, r.partials, r.ticket, gnorm2, phi);
             return cudaGetLastError();

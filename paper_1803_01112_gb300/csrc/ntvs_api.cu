@@ -142,6 +142,7 @@ struct ntvs_ctx {
     float* xh = nullptr;   // FP32 path: fl32(x) and fl32(x - xh), canonical order (TV stencil)
     float* xl = nullptr;
     void* delta = nullptr;
+    int delta_copies = 1;              // FP64: arrays of delta that a block's rows scatter into (see below)
     void* g = nullptr;
     RedScratch red{nullptr, nullptr, 1};
     double* dscal = nullptr;   // [0] ||g||^2, [1] phi(x), [2] phi(z), [3] phi for ntvs_get_tv
@@ -534,7 +535,7 @@ int perturb_steps(ntvs_ctx* c, int64_t* ell_io) {
 // (nothing applied), its residual sum of squares into *resid.  The whole block runs the
 // context's schedule; a proper sub-range of it runs the plain schedule (the windowed and
 // pipelined plans cover whole blocks).
-int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid) {
+int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid, int copies = 1) {
     if (r1 <= r0) return NTVS_OK;
     const bool whole = r0 == c->block_ptr[t] && r1 == c->block_ptr[t + 1];
     if (c->paths_mode) {
@@ -554,6 +555,8 @@ int launch_drop_kernel(ntvs_ctx* c, int t, int64_t r0, int64_t r1, double* resid
     a.r1 = r1;
     a.x = (c->cdt == F64) ? (const void*)c->x : (const void*)c->x32;
     a.delta = c->delta;
+    a.copies = copies;
+    a.delta_stride = c->vm.vint;
     a.lambda = c->p.lambda;
     a.resid_ss = resid;
     a.vdt = c->vdt;
@@ -618,7 +621,9 @@ int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
     if (!resid_cleared) CUDA_TRY(cudaMemsetAsync(c->resid + t, 0, sizeof(double), c->stream));
     if (r1 <= r0 && !c->ar_fn) return NTVS_OK;
     const bool windowed = r1 > r0 && c->schedule == NTVS_SCHED_WINDOW && c->segs;
-    TRY(launch_drop_kernel(c, t, r0, r1, c->resid + t));
+    // ranks sum delta itself, and the pipelined schedule writes it
+    const int copies = c->ar_fn || c->schedule == NTVS_SCHED_PIPELINE ? 1 : c->delta_copies;
+    TRY(launch_drop_kernel(c, t, r0, r1, c->resid + t, copies));
     if (c->ar_fn) {
         int rc = c->ar_fn(c->delta, c->vm.vint, c->cdt, (void*)c->stream, c->ar_user);
         if (rc == 0) rc = c->ar_fn(c->resid + t, 1, NTVS_F64, (void*)c->stream, c->ar_user);
@@ -627,6 +632,9 @@ int drop_block(ntvs_ctx* c, int t, bool resid_cleared = false) {
                                            std::to_string(rc) + ")");
     }
     CUDA_TRY(timed_launch(c, KIND_APPLY, [&] {
+        if (copies > 1)
+            return k_drop_apply_copies(c->x, (double*)c->delta, copies, c->vm.vint,
+                                       (const double*)c->inv_s + (size_t)t * c->vm.vint, c->V, c->stream);
         return k_drop_apply(c->cdt, c->x, c->copies(split), c->delta,
                             (const char*)c->inv_s + (size_t)t * c->vm.vint * c->csz(), c->V, c->apply_grid,
                             windowed ? c->wlog : nullptr, c->win_grid, r1 - r0,
@@ -716,6 +724,21 @@ static int pack_delta16(ntvs_ctx* c) {
         c->own_val = false;
     }
     return NTVS_OK;
+}
+
+// ---- FP64 scatter copies ---------------------------------------------------------------------
+// FP64 rows scatter with global reductions, and many rows on few voxels queue at the L2 for the
+// same addresses.  Then the CTAs scatter into several copies of delta, which the apply sums.  us a
+// sweep with 1 / 4 / 16 copies, by a block's entries a voxel (FP64 rows in detected order):
+//   16x16x1   138: 136 / 107 / 127    1719: 1339 / 532 / 455    11458: 1157 / 340 / 207
+//   32x32x1    69: 111 / 107 / 127     859: 900 / 522 / 513      5729: 1071 / 335 / 237
+//   41x41x1   179: 54 / 48 / 54        671: 784 / 706 / 686      4472: 571 / 423 / 424
+//   96x96x1   115: 254 / 250 / 263     286: 826 / 829 / 828      1910: 525 / 507 / 508
+//   96x96x8    36: 1148 / 1273 / 1335  239: 908 / 860 / 870
+// (In binned order the same within a few per cent.)
+static int fp64_delta_copies(int64_t voxels, int64_t entries) {
+    const int64_t hits = voxels > 0 ? entries / voxels : 0;
+    return voxels > 65536 || hits < 100 ? 1 : hits < 800 ? 4 : 16;
 }
 
 // ---- DROP schedule planning (load time) ------------------------------------------------
@@ -846,9 +869,10 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
 
     // FP64 arithmetic: the windowed schedule runs without the window.  A shared-memory FP64 add
     // is a compare-and-swap loop, a global one is native, and rows in stored order with global
-    // reductions measured faster at every size that has a window (us per block, global against
-    // window: 10.4 / 20.9 at 2000 rows of 32x32x1, 28.6 / 33.0 at 8000 and 218 / 260 at 120000
-    // rows of 96x96x12).
+    // reductions (into copies of delta where many rows share few voxels, fp64_delta_copies)
+    // measured faster wherever there is a window (us per block, global against window: 10.4 / 20.9 at
+    // 2000 rows of 32x32x1, 79 / 121 at 166 667, 28.6 / 33.0 at 8000 and 218 / 260 at 120000 rows of
+    // 96x96x12).
     if (c->cdt == F64 && requested != NTVS_SCHED_PIPELINE) {
         c->schedule = NTVS_SCHED_WINDOW;
         return NTVS_OK;
@@ -1371,14 +1395,15 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
         TRY(dev_alloc(&c->xh, sizeof(float) * (size_t)V, "xh"));
         TRY(dev_alloc(&c->xl, sizeof(float) * (size_t)V, "xl"));
     }
-    TRY(dev_alloc(&c->delta, csz * (size_t)VI, "delta"));
+    c->delta_copies = c->cdt == F64 ? fp64_delta_copies(VI, nnz / std::max(c->B, 1)) : 1;
+    TRY(dev_alloc(&c->delta, csz * (size_t)VI * c->delta_copies, "delta"));
     TRY(dev_alloc(&c->g, csz * (size_t)V, "g"));
     TRY(dev_alloc(&c->resid, sizeof(double) * (size_t)c->B, "residuals"));
     CUDA_TRY(cudaMemsetAsync(c->x, 0, sizeof(double) * (size_t)V, st));
     if (c->x32) CUDA_TRY(cudaMemsetAsync(c->x32, 0, sizeof(float) * (size_t)VI, st));
     if (c->xh) CUDA_TRY(cudaMemsetAsync(c->xh, 0, sizeof(float) * (size_t)V, st));
     if (c->xl) CUDA_TRY(cudaMemsetAsync(c->xl, 0, sizeof(float) * (size_t)V, st));
-    CUDA_TRY(cudaMemsetAsync(c->delta, 0, csz * (size_t)VI, st));
+    CUDA_TRY(cudaMemsetAsync(c->delta, 0, csz * (size_t)VI * c->delta_copies, st));
     CUDA_TRY(cudaMemsetAsync(c->g, 0, csz * (size_t)V, st));
     CUDA_TRY(cudaMemsetAsync(c->resid, 0, sizeof(double) * (size_t)c->B, st));
 

@@ -215,6 +215,8 @@ struct DropArgs {
     int64_t r0, r1;
     const void* x;         // gather image: FP64 master (F64 path) or its FP32 copy (F32 path)
     void* delta;           // compute type, accumulates lambda * sum_i a_ij r_i
+    int copies;            // FP64 plain schedule: CTA c scatters into copy c % copies of delta, delta_stride
+    int64_t delta_stride;  // values apart (1: delta itself)
     double lambda;
     double* resid_ss;      // += sum_i (b_i - <a_i,x>)^2
     int vdt, cdt;
@@ -291,6 +293,9 @@ cudaError_t k_chunk_home(const int32_t* home, const int64_t* chunk_start, int64_
 cudaError_t k_drop_apply(int cdt, double* x, ImgCopies c, void* delta, const void* inv_s, int64_t V, int grid,
                          const float* wlog, int ctas, int64_t rows, float* rms, cudaStream_t s);
 
+// the same on the FP64 path (canonical order, no FP32 copies) with delta the sum of `copies` arrays
+cudaError_t k_drop_apply_copies(double* x, double* delta, int copies, int64_t delta_stride, const double* inv_s,
+                                int64_t V, cudaStream_t s);
 // TMA-fed pipeline (drop_pipe_kernel): a stage is a run of at most kStageRows whole rows
 // of one home slice whose entries [e0, e0 + nent) fit one ring slot (e0 and nent aligned
 // to 16 bytes of both col and val); off[k] = row_ptr[r0 + k] - e0.  nent == 0 marks a
