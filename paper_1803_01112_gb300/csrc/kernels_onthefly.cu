@@ -283,24 +283,30 @@ constexpr int kOtfThreads = 256;
 constexpr int kOtfWarps = kOtfThreads / 32;
 
 // Entries of a warp's buffer, from two rows' pieces on the grid's diagonal (every plane of x and y
-// crossed; straight in z) with their segment joins: 54 KB a CTA and four CTAs an SM, or 72 KB and
-// three, 114 KB and two, 225 KB and one.  Rows off the diagonal have fewer pieces (1.27 n on
-// average on n x n voxels, against 2 n), so a size serves grids somewhat past its diagonal; what
-// does not fit is walked twice, and slowest by far.  Sweeps of 400k rows of 16 segments with
-// three / two / one CTA, us (24 cached pieces a lane, before the buffer: last number):
+// crossed; straight in z) with their segment joins: 54 or 72 KB a CTA and three CTAs an SM, 114 KB
+// and two, or 225 KB and one.  Rows off the diagonal have fewer pieces (1.27 n on average on n x n voxels,
+// against 2 n), so a size serves grids somewhat past its diagonal; what does not fit is walked twice.
+// Where most rows do not, a few entries serve as well, with three CTAs and the L1 for the image: 1536x1536,
+// 400k rows 5271 us with one CTA and 3773 so (4766 before the buffer), 1024x1024x2 3053 / 2979, 896x896x4
+// 2668 / 2881.  Keeping the segments of such a row that fit, the others walked twice, was slower than
+// either (5692 us on 2048x2048; 4516 / 2794) and cost the others 8 %.  Sweeps of 400k rows of 16 segments with three / two / one CTA, us (24 cached
+// pieces a lane, before the buffer: last number):
 //   256x256x16  669 / 704 / 1099 (1088)     512x512x16  2410 / 1483 / 1878 (2379)
 //   320x320x16  913 / 837 / 1295 (1413)     576x576x16  3050 / 1962 / 2064 (2745)
 //   448x448x16  1837 / 1142 / 1691 (2059)   640x640x8   2945 / 2352 / 2092 (2833)
 //   1024x256x8  1886 / 1554 / 1666 (2019)   1024x1024x4 4566 / 4175 / 3253 (4302)
+// Four CTAs, which fit with smaller buffers on small grids, spill: 64x64x8, 100k rows of 16 / 24
+// segments, 155 / 205 us with four and 129 / 170 with three (152 / 173 before the buffer).
 struct OtfBuffer {
     int entries, ctas;   // per warp; CTAs an SM
 };
 static OtfBuffer otf_buffer(const OtfArgs& a) {
     const int64_t need = 2 * ((int64_t)a.nx + a.ny + 2 * a.n_seg + 8);
-    if (need <= 864) return {864, 4};
+    if (need <= 864) return {864, 3};
     if (need <= 1136) return {1136, 3};
     if (need <= 2500) return {1776, 2};
-    return {3520, 1};
+    if (need <= 4100) return {3520, 1};
+    return {64, 3};   // no buffer to speak of
 }
 
 template <int MINB>
@@ -531,7 +537,7 @@ cudaError_t k_otf_drop(const OtfArgs& a, int64_t r0, int64_t r1, const float* in
     if (r1 <= r0) return cudaSuccess;
     const OtfBuffer buf = otf_buffer(a);
     const size_t smem = (size_t)buf.entries * kOtfWarps * sizeof(int2);
-    auto kern = buf.ctas == 4 ? otf_drop_kernel<4> : buf.ctas == 3 ? otf_drop_kernel<3> : otf_drop_kernel<2>;
+    auto kern = buf.ctas == 3 ? otf_drop_kernel<3> : otf_drop_kernel<2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = a.grid / 8 * buf.ctas;   // a.grid: 8 CTAs per SM; one resident wave

@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
     (520, 510, 2, 16, 701),      # two CTAs an SM: rows near the diagonal overflow
     (640, 600, 1, 16, 601),      # one CTA an SM: everything fits
     (1000, 950, 1, 16, 601),     # rows near the diagonal overflow it
+    (1100, 1000, 1, 16, 401),    # no buffer: every row is walked twice
 ])
 def test_traced_delta_on_wide_grids(nx, ny, nz, n_seg, n_hist):
     ntvs = ntvs_module()
