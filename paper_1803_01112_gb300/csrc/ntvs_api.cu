@@ -60,6 +60,14 @@ int dev_alloc(T** p, size_t bytes, const char* what) {
     return NTVS_OK;
 }
 
+// an allocation that may fail (for what has a fallback): false, and *p null, without room
+template <typename T>
+bool dev_try(T** p, size_t bytes) {
+    if (cudaMalloc((void**)p, bytes) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    *p = nullptr;
+    return false;
+}
 template <typename T>
 void dev_free(T*& p) {
     if (p) cudaFree((void*)p);
@@ -849,13 +857,17 @@ static int plan_schedule(ntvs_ctx* c, int requested) {
         if (!c->ent || c->cdt != F32 || c->win_lpr < 16 || c->nz > kOrderHomes || c->M > INT32_MAX ||
             longest > INT32_MAX || c->nnz / std::max(c->B, 1) < kOrderEntries)   // 32-bit rows and lengths
             return NTVS_OK;
-        TRY(dev_alloc(&c->order, sizeof(int32_t) * (size_t)c->M, "row order"));
+        // without room for the index (8 bytes a row) the rows keep the plain schedule, which needs none
         int32_t* dsorted = nullptr;
-        TRY(dev_alloc(&dsorted, sizeof(int32_t) * (size_t)c->M, "ordered home slices"));
         struct FreeSorted {
             int32_t*& p;
             ~FreeSorted() { dev_free(p); }
         } sorted_guard{dsorted};
+        if (!dev_try(&c->order, sizeof(int32_t) * (size_t)c->M)) return NTVS_OK;
+        if (!dev_try(&dsorted, sizeof(int32_t) * (size_t)c->M)) {
+            dev_free(c->order);
+            return NTVS_OK;
+        }
         CUDA_TRY(cudaMemcpyAsync(dbp, c->block_ptr.data(), sizeof(int64_t) * ((size_t)c->B + 1), cudaMemcpyHostToDevice,
                                  c->stream));
         CUDA_TRY(k_order_rows(dhome, dbp, c->B, c->nz, c->order, dsorted, c->stream));
@@ -1400,7 +1412,8 @@ int ntvs_load_system(ntvs_ctx* c, const ntvs_system* s) {
         TRY(dev_alloc(&c->xl, sizeof(float) * (size_t)V, "xl"));
     }
     c->delta_copies = c->cdt == F64 ? fp64_delta_copies(VI, nnz / std::max(c->B, 1)) : 1;
-    TRY(dev_alloc(&c->delta, csz * (size_t)VI * c->delta_copies, "delta"));
+    if (c->delta_copies > 1 && !dev_try(&c->delta, csz * (size_t)VI * c->delta_copies)) c->delta_copies = 1;
+    if (!c->delta) TRY(dev_alloc(&c->delta, csz * (size_t)VI, "delta"));
     TRY(dev_alloc(&c->g, csz * (size_t)V, "g"));
     TRY(dev_alloc(&c->resid, sizeof(double) * (size_t)c->B, "residuals"));
     CUDA_TRY(cudaMemsetAsync(c->x, 0, sizeof(double) * (size_t)V, st));
